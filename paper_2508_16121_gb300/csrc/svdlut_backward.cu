@@ -9,8 +9,9 @@
 //                warp-private tables G_p[i][j][c] (one LUT pair, all three
 //                output channels per warp: one key match per pixel and pair),
 //                then sums the warps of a CTA into a per-CTA partial.
-//   3. grid    : grid_grad_kernel does the same for the folded grid planes
-//                (xy, xc, yc per output channel) over 128-px column blocks.
+//   3. grid    : grid_grad_kernel sums the folded grid planes (xy, xc, yc per
+//                output channel) over 128-px column blocks, in lane-private
+//                bins.
 //   4. reduce  : lut_finalize_kernel sums the CTA partials and contracts
 //                through T = U diag(S) V^T (Eq. 9) to dU, dS, dV, dlut_w;
 //                grid_reduce_kernel sums the block partials per vertex into dg_*
@@ -266,47 +267,102 @@ __global__ void __launch_bounds__(kLutThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// grid gradients per output channel c (folded planes F_c = sum_{k=c mod 3}
-// w_k g_k): dFxy_c[iy][ix], dFxc_c[ix][j], dFyc_c[iy][j] = scatters of dy_c.
-// Blocks: 128-px column strip x BH rows (host plan); warp w owns a contiguous
-// run of rows.  Output per block: xy [nvy][nvx][3], xc [3][nvx][Dsc],
-// yc [3][nvy][Dsc] in block-local indexing.
+// Grid gradients per output channel c (folded planes F_c = sum_{k=c mod 3}
+// w_k g_k): dFxy_c[iy][ix], dFxc_c[ix][j], dFyc_c[iy][j].
+// Blocks: 128-px column strip x BH rows (host plan); warp (group g, channel c)
+// owns a contiguous run of rows of one channel.  Output per block: xy
+// [nvy][nvx][3], xc [3][nvx][Dsc], yc [3][nvy][Dsc] in block-local indexing.
+//
+// All three planes of a channel spread the same two numbers per pixel, v0 =
+// dy (1 - e) at intensity vertex j and v1 = dy e at j + 1.  A lane owns four
+// adjacent columns of the strip and walks down its warp's rows, so
+//   xc: a column's x weights are fixed; its sums over the rows go to the
+//       column's own bins X[j][column] and are spread over the x vertices once
+//       per block;
+//   yc: the rows of one y-cell share their two vertices; the lane adds
+//       (v (1 - dy), v dy) to its own bins Y[j][lane], which are summed over
+//       the lanes when the y-cell changes;
+//   xy: sum dy_c (1 - dy) and sum dy_c dy stay in registers per column and
+//       are spread over the x vertices when the y-cell changes.
+// The bank of every bin is the lane's own, so the updates are conflict-free
+// and need no match, tree or barrier; every sum has one owner and a fixed
+// order (bitwise repeatable).  Two y moments (not one bin row per image row)
+// keep the lane sums off the per-row path; four columns per lane share one Y.
+// One channel per warp, because a warp's bins (13 KB at Dsc = 17) bound the
+// warps of an SM: 15 warps, where warps of three channels left 5 and the
+// kernel waited on its own latency (361 us on 8 x 1920x1080).
+// Measured on 8 x 1920x1080, grids at 1/8 resolution: 204 us, the shared-memory
+// pipe at 56 % and the issue slots at 50 %; 655 us when each pixel went through
+// a warp scatter (match, rank tree, leader's update) per channel.
 // ---------------------------------------------------------------------------
 struct GridPlan {
     int BH, bands, nblk;   // per image
     int nvx, nvy, rpw, nvyw;  // maxima
     int blk_stride;        // floats per block partial
-    int bins;              // 1: yc through lane-private bins, 0: warp scatter (large Dsc)
+    int groups;            // row groups of a block (one warp per channel each)
 };
-
-// Per-warp floats: the xy, xc and yc tables, then the lane-private yc bins
-// [3][Dsc][33] (one column per lane, padded so that a lane summing a row of
-// bins reads 32 different banks).
-__host__ __device__ inline int grid_table_floats(int nvx, int nvyw, int Dsc)
-{
-    return (3 * nvyw * nvx + 3 * nvx * Dsc + 3 * nvyw * Dsc + 3) & ~3;
-}
-__host__ __device__ inline int grid_warp_floats(int nvx, int nvyw, int Dsc, int bins)
-{
-    return grid_table_floats(nvx, nvyw, Dsc) + (bins ? 3 * Dsc * 33 : 0);
-}
 
 __host__ __device__ inline int grid_block_floats(int nvx, int nvy, int Dsc)
 {
     return 3 * nvy * nvx + 3 * nvx * Dsc + 3 * nvy * Dsc;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+constexpr int kGridGroups = 5;
+constexpr int kGridThreads = 3 * kGridGroups * 32;
+
+// floats of one warp: Y (at least the 2 x 128 staging of the xy flush), X,
+// then the warp's yc and xy vertex rows
+__host__ __device__ inline int grid_y_floats(int Dsc) { return Dsc * 64 > 2 * kTileW ? Dsc * 64 : 2 * kTileW; }
+__host__ __device__ inline int grid_warp_floats(int nvx, int nvyw, int Dsc)
+{
+    return grid_y_floats(Dsc) + Dsc * kTileW + ((nvyw * (Dsc + nvx) + 3) & ~3);
+}
+// floats shared by the block: column offsets, first column of each x-cell
+__host__ __device__ inline int grid_shared_floats(int nvx) { return kTileW + ((nvx + 1 + 3) & ~3); }
+
+// Sums of 128 per-column values (column col at (col & 3) * 32 + (col >> 2))
+// over the x vertices of the block: vertex v takes the columns of cell v with
+// weight 1 - d and those of cell v - 1 with weight d.  Lanes are (part,
+// vertex) pairs: each adds a contiguous part of its vertex's columns in order,
+// the parts are combined by a butterfly.  store(v, sum) is called by part 0.
+template <class Store>
+__device__ __forceinline__ void spread_columns(const float *row, const float *cold, const int *cs, int nvx,
+                                               Store store)
+{
+    const int lane = threadIdx.x & 31;
+    int nvp = 2;
+    while (nvp < nvx && nvp < 32) nvp <<= 1;
+    const int parts = 32 / nvp, part = lane / nvp;
+    for (int v0 = 0; v0 < nvx; v0 += nvp) {
+        const int v = v0 + (lane & (nvp - 1));
+        float s = 0.f;
+        if (v < nvx) {
+            const int lo = cs[max(v - 1, 0)], mid = cs[v], hi = cs[min(v + 1, nvx)];
+            const int len = (hi - lo + parts - 1) / parts;
+            const int c0 = lo + part * len, c1 = min(c0 + len, hi);
+            for (int col = c0; col < c1; ++col) {
+                const float d = cold[col], w = col < mid ? d : 1.f - d;
+                s = fmaf(row[(col & 3) * 32 + (col >> 2)], w, s);
+            }
+        }
+        for (int o = nvp; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (part == 0 && v < nvx) store(v, s);
+    }
+}
+
+__global__ void __launch_bounds__(kGridThreads, 1)
     grid_grad_kernel(BwdArgs a, GridPlan gp, float *__restrict__ grid_part)
 {
     extern __shared__ __align__(16) float sm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ int wy_off[kGridGroups], wy_n[kGridGroups];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = gp.groups * 3, nthr = nw * 32;
+    const int grp = warp / 3, c = warp - grp * 3;
     const int b = blockIdx.y, lb = blockIdx.x;
     const int band = lb / a.strips, strip = lb - band * a.strips;
     const int x0 = strip * kTileW, y0 = band * gp.BH;
     const int rows = min(gp.BH, a.H - y0);
     if (rows <= 0) return;
-    const int Dsc = a.Dsc, Dc2 = Dsc - 2;
+    const int Dsc = a.Dsc;
     // block footprint
     int ixlo, ixhi, iylo, iyhi;
     float t;
@@ -317,8 +373,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int nvx = min(min(ixhi + 1, a.Dsx - 1) - ixlo + 1, gp.nvx);
     const int nvy = min(min(iyhi + 1, a.Dsy - 1) - iylo + 1, gp.nvy);
     // this warp's rows and their footprint
-    const int rpw = (rows + kWarps - 1) / kWarps;
-    const int wr0 = min(warp * rpw, rows), wr1 = min(wr0 + rpw, rows);
+    const int rpw = (rows + gp.groups - 1) / gp.groups;
+    const int wr0 = min(grp * rpw, rows), wr1 = min(wr0 + rpw, rows);
     int wylo = iylo, wyhi = iylo;
     if (wr1 > wr0) {
         spatial_cell(y0 + wr0, a.H, a.Dsy, a.rH1, wylo, t);
@@ -326,162 +382,240 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     const int nvyw = min(min(wyhi + 1, a.Dsy - 1) - wylo + 1, gp.nvyw);
 
-    const int wf = grid_warp_floats(gp.nvx, gp.nvyw, Dsc, gp.bins);
-    float *wt = sm + warp * wf;
-    float *txy = wt;                             // [nvyw][nvx][3]
-    float *txc = txy + 3 * gp.nvyw * gp.nvx;     // [3][nvx][Dsc]
-    float *tyc = txc + 3 * gp.nvx * Dsc;         // [3][nvyw][Dsc]
-    float *hb = wt + grid_table_floats(gp.nvx, gp.nvyw, Dsc);  // [3][Dsc][33] yc bins of this row
-    for (int e = threadIdx.x; e < kWarps * wf; e += kThreads) sm[e] = 0.f;
-    __syncthreads();
+    float *cold = sm;                                // [kTileW]
+    int *cs = reinterpret_cast<int *>(sm + kTileW);  // [nvx + 1]
+    float *wbase = sm + grid_shared_floats(gp.nvx);
+    const int wf = grid_warp_floats(gp.nvx, gp.nvyw, Dsc);
+    const int yf = grid_y_floats(Dsc), xf = Dsc * kTileW;
+    float *wt = wbase + warp * wf;
+    float2 *Y = reinterpret_cast<float2 *>(wt);  // [Dsc][32 lanes]
+    float *X = wt + yf;                          // [Dsc][4 x 32 columns]
+    float *tyc = X + xf;                         // [nvyw][Dsc]
+    float *txy = tyc + gp.nvyw * Dsc;            // [nvyw][nvx]
+    for (int e = threadIdx.x; e < nw * wf / 4; e += nthr)
+        reinterpret_cast<float4 *>(wbase)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // column offsets and the first column of each x-cell (cells 0 .. nvx - 2)
+    const int ncols = min(kTileW, a.W - x0);
+    for (int col = threadIdx.x; col < ncols; col += nthr) {
+        int ix, ixp = -1;
+        float d, dp;
+        spatial_cell(x0 + col, a.W, a.Dsx, a.rW1, ix, d);
+        ix = max(0, min(ix - ixlo, nvx - 2));
+        if (col > 0) {
+            spatial_cell(x0 + col - 1, a.W, a.Dsx, a.rW1, ixp, dp);
+            ixp = max(0, min(ixp - ixlo, nvx - 2));
+        }
+        cold[col] = d;
+        for (int v = ixp + 1; v <= ix; ++v) cs[v] = col;
+        if (col == ncols - 1)
+            for (int v = ix + 1; v <= nvx; ++v) cs[v] = ncols;
+    }
 
     const size_t plane = static_cast<size_t>(a.H) * a.W;
-    const float *xb = a.x + static_cast<size_t>(b) * 3 * plane;
-    const float *gb = a.dy + static_cast<size_t>(b) * 3 * plane;
-    const float fS1 = static_cast<float>(Dsc - 1), fS2 = static_cast<float>(Dc2);
     const int x = x0 + lane * 4;
     const int n = min(4, a.W - x);
-    int ixl[4];
-    float dxk[4];
+    const float *xb = a.x + (static_cast<size_t>(b) * 3 + c) * plane + x;
+    const float *gb = a.dy + (static_cast<size_t>(b) * 3 + c) * plane + x;
+    const bool vec = a.vec && n == 4;
+    const float fS1 = static_cast<float>(Dsc - 1), fS2 = static_cast<float>(Dsc - 2);
+    // The lane's columns, and whether every lane's lie in at most two x-cells:
+    // then a column adds to vertices i0 + cell and i0 + cell + 1, cell 0 or 1.
+    float cd[4];
+    bool c1[4];
+    int i0 = 0, i3 = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         int ix;
-        spatial_cell(min(x + k, a.W - 1), a.W, a.Dsx, a.rW1, ix, dxk[k]);
-        ixl[k] = max(0, min(ix - ixlo, nvx - 2));
+        spatial_cell(min(x + k, a.W - 1), a.W, a.Dsx, a.rW1, ix, cd[k]);
+        if (k == 0) i0 = ix;
+        c1[k] = ix != i0;
+        i3 = ix;
     }
-    // xy: the weights factor as (y part) x (x part) and a lane's columns are
-    // fixed, so sum_rows dy_c (1 - dy) and sum_rows dy_c dy are kept per
-    // pixel while the rows stay in one y-cell and scattered when it changes.
-    float sy0[4][3], sy1[4][3];
+    const bool two_cells = __all_sync(0xffffffffu, i3 - i0 <= 1);
+    __syncthreads();
+
+    float sy0[4], sy1[4];  // xy sums of this lane's columns in the current y-cell
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sy0[k][c] = sy1[k][c] = 0.f;
-    int iyw_acc = -1;
-    auto flush_xy = [&]() {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float dx = dxk[k];
-            float v[4][3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                v[0][c] = sy0[k][c] * (1.f - dx);
-                v[1][c] = sy1[k][c] * (1.f - dx);
-                v[2][c] = sy0[k][c] * dx;
-                v[3][c] = sy1[k][c] * dx;
-                sy0[k][c] = sy1[k][c] = 0.f;
+    for (int k = 0; k < 4; ++k) sy0[k] = sy1[k] = 0.f;
+    // end of a y-cell (warp row iyw): Y over the lanes into tyc, the xy sums
+    // over the columns into txy, both cleared
+    auto flush = [&](int iyw) {
+        __syncwarp();
+        // an entry's lane sum starts at pair e mod 16 of the lanes and wraps:
+        // neighbouring entries read different banks at a time
+        for (int e = lane; e < Dsc; e += 32) {
+            const float4 *row = reinterpret_cast<const float4 *>(Y) + e * 16;
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+            for (int l = 0; l < 16; ++l) {
+                const float4 q = row[(l + e) & 15];
+                s0 += q.x + q.z;
+                s1 += q.y + q.w;
             }
-            warp_scatter<3>(txy, k < n ? (iyw_acc * gp.nvx + ixl[k]) * 3 : -1, gp.nvx * 3, 3, v);
+            float *t0 = tyc + iyw * Dsc + e;
+            t0[0] += s0;
+            t0[Dsc] += s1;
+        }
+        __syncwarp();
+        float *r0 = txy + iyw * gp.nvx, *r1 = r0 + gp.nvx;
+        if (two_cells) {
+            // the lane's sums at vertices i0, i0 + 1 and i0 + 2, then every
+            // vertex adds those of the lanes that touch it, in order
+            float2 s[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float w1 = cd[k], w0 = 1.f - w1;
+                const float2 lo = make_float2(sy0[k] * w0, sy1[k] * w0), hi = make_float2(sy0[k] * w1, sy1[k] * w1);
+                const int q = c1[k] ? 1 : 0;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    if (i == q) s[i] = make_float2(s[i].x + lo.x, s[i].y + lo.y);
+                    if (i == q + 1) s[i] = make_float2(s[i].x + hi.x, s[i].y + hi.y);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) Y[q * 32 + lane] = s[q];
+            __syncwarp();
+            for (int v = lane; v < nvx; v += 32) {
+                float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int i = v - q;  // lanes whose first column lies in cell i
+                    if (i < 0 || i > nvx - 2) continue;
+                    for (int l = (cs[i] + 3) >> 2; l < (cs[i + 1] + 3) >> 2; ++l) {
+                        const float2 u = Y[q * 32 + l];
+                        s0 += u.x;
+                        s1 += u.y;
+                    }
+                }
+                r0[v] += s0;
+                r1[v] += s1;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                wt[k * 32 + lane] = sy0[k];
+                wt[kTileW + k * 32 + lane] = sy1[k];
+            }
+            __syncwarp();
+            spread_columns(wt, cold, cs, nvx, [&](int v, float s) { r0[v] += s; });
+            __syncwarp();
+            spread_columns(wt + kTileW, cold, cs, nvx, [&](int v, float s) { r1[v] += s; });
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sy0[k] = sy1[k] = 0.f;
+        __syncwarp();
+        for (int e = lane; e < yf / 4; e += 32) reinterpret_cast<float4 *>(wt)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncwarp();
+    };
+
+    auto load = [&](int r, float4 &p, float4 &g) {
+        p = g = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < wr1 && n > 0) {
+            const size_t off = static_cast<size_t>(y0 + r) * a.W;
+            p = PixIO<float>::load(xb + off, n, vec);
+            g = PixIO<float>::load(gb + off, n, vec);
         }
     };
-    for (int r = wr0; r < wr1; ++r) {
-        const int y = y0 + r;
-        int iy;
-        float dy;
-        spatial_cell(y, a.H, a.Dsy, a.rH1, iy, dy);
-        const int iyw = max(0, min(iy - wylo, nvyw - 2));
-        if (iyw != iyw_acc) {
-            if (iyw_acc >= 0) flush_xy();
-            iyw_acc = iyw;
+    int iy_acc = -1, cy = 0;
+    float cdy = 0.f;
+    auto row = [&](int r, const float4 &p, const float4 &g4) {
+        // y-cells of the next 32 rows, one per lane
+        const int ri = (r - wr0) & 31;
+        if (ri == 0) {
+            spatial_cell(min(y0 + r + lane, a.H - 1), a.H, a.Dsy, a.rH1, cy, cdy);
+            cy = max(0, min(cy - wylo, nvyw - 2));
         }
-        const size_t o = static_cast<size_t>(y) * a.W + x;
-        float4 P[3], G[3];
+        const int iyw = __shfl_sync(0xffffffffu, cy, ri);
+        const float dy = __shfl_sync(0xffffffffu, cdy, ri), dy0 = 1.f - dy;
+        if (iyw != iy_acc) {
+            if (iy_acc >= 0) flush(iy_acc);
+            iy_acc = iyw;
+        }
+        int j[4];
+        float v0[4], v1[4], u0[4], u1[4];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            P[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-            G[c] = P[c];
-            if (n > 0) {
-                P[c] = PixIO<float>::load(xb + c * plane + o, n, a.vec && n == 4);
-                G[c] = PixIO<float>::load(gb + c * plane + o, n, a.vec && n == 4);
-            }
+        for (int k = 0; k < 4; ++k) {
+            const float g = get(g4, k);
+            float e;
+            j[k] = cell_of(__saturatef(get(p, k)), fS1, fS2, e);
+            v0[k] = g * (1.f - e);
+            v1[k] = g * e;
+            sy0[k] = fmaf(g, dy0, sy0[k]);
+            sy1[k] = fmaf(g, dy, sy1[k]);
+            const float *xp = X + j[k] * kTileW + k * 32 + lane;
+            u0[k] = xp[0];
+            u1[k] = xp[kTileW];
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const bool act = k < n;
-            const float dx = dxk[k];
-            float gy[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) gy[c] = act ? get(G[c], k) : 0.f;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {  // xy corners (iy, ix), (iy+1, ix), (iy, ix+1), (iy+1, ix+1)
-                sy0[k][c] = fmaf(gy[c], 1.f - dy, sy0[k][c]);
-                sy1[k][c] = fmaf(gy[c], dy, sy1[k][c]);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float pc = fminf(fmaxf(get(P[c], k), 0.f), 1.f);
-                float ec;
-                const int jc = cell_of(pc, fS1, fS2, ec);
-                {   // xc: corners (ix, j), (ix+1, j), (ix, j+1), (ix+1, j+1)
-                    float v[4][1] = {{gy[c] * (1.f - dx) * (1.f - ec)}, {gy[c] * dx * (1.f - ec)},
-                                     {gy[c] * (1.f - dx) * ec}, {gy[c] * dx * ec}};
-                    warp_scatter<1>(txc + c * gp.nvx * Dsc, act ? ixl[k] * Dsc + jc : -1, Dsc, 1, v);
-                }
-                if (gp.bins) {
-                    // yc: the row (hence dy and the y-cell) is common to the warp, so
-                    // the intensity weights go to this lane's own bins (no conflicts)
-                    // and are spread over the corners (iy, iy+1) once per row
-                    hb[(c * Dsc + jc) * 33 + lane] += gy[c] * (1.f - ec);
-                    hb[(c * Dsc + jc + 1) * 33 + lane] += gy[c] * ec;
-                } else {  // yc: corners (iy, j), (iy+1, j), (iy, j+1), (iy+1, j+1)
-                    float v[4][1] = {{gy[c] * (1.f - dy) * (1.f - ec)}, {gy[c] * dy * (1.f - ec)},
-                                     {gy[c] * (1.f - dy) * ec}, {gy[c] * dy * ec}};
-                    warp_scatter<1>(tyc + c * gp.nvyw * Dsc, act ? iyw * Dsc + jc : -1, Dsc, 1, v);
-                }
-            }
+            float *xp = X + j[k] * kTileW + k * 32 + lane;
+            xp[0] = u0[k] + v0[k];
+            xp[kTileW] = u1[k] + v1[k];
         }
-        // yc bins of this row: lane-ordered sums, spread over rows iy, iy+1
-        __syncwarp();
-        for (int e = lane; gp.bins && e < 3 * Dsc; e += 32) {
-            float *col = hb + e * 33;
-            float sum = 0.f;
-#pragma unroll 8
-            for (int l = 0; l < 32; ++l) {
-                sum += col[l];
-                col[l] = 0.f;
-            }
-            const int c = e / Dsc, j = e - c * Dsc;
-            float *t0 = tyc + (c * gp.nvyw + iyw) * Dsc + j;
-            t0[0] = fmaf(1.f - dy, sum, t0[0]);
-            t0[Dsc] = fmaf(dy, sum, t0[Dsc]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float2 *yp = Y + j[k] * 32 + lane;
+            const float2 q0 = yp[0], q1 = yp[32];
+            yp[0] = make_float2(fmaf(v0[k], dy0, q0.x), fmaf(v0[k], dy, q0.y));
+            yp[32] = make_float2(fmaf(v1[k], dy0, q1.x), fmaf(v1[k], dy, q1.y));
         }
-        __syncwarp();
+    };
+    float4 pa, ga, pb, gb4;
+    load(wr0, pa, ga);
+    for (int r = wr0; r < wr1; r += 2) {
+        load(r + 1, pb, gb4);
+        row(r, pa, ga);
+        load(r + 2, pa, ga);
+        if (r + 1 < wr1) row(r + 1, pb, gb4);
     }
-    if (iyw_acc >= 0) flush_xy();
-    // the warps' first vertex row relative to the block's
-    __shared__ int wy_off[kWarps], wy_n[kWarps];
-    if (lane == 0) {
-        wy_off[warp] = wylo - iylo;
-        wy_n[warp] = wr1 > wr0 ? nvyw : 0;
+    if (iy_acc >= 0) flush(iy_acc);
+    if (lane == 0 && c == 0) {
+        wy_off[grp] = wylo - iylo;
+        wy_n[grp] = wr1 > wr0 ? nvyw : 0;
     }
     __syncthreads();
-    // block partial: sum the warps in order (each block entry independently)
+    // block partial: the row groups in order
     float *out = grid_part + (static_cast<size_t>(b) * gp.nblk + lb) * gp.blk_stride;
     float *oxy = out, *oxc = out + 3 * gp.nvy * gp.nvx, *oyc = oxc + 3 * gp.nvx * Dsc;
-    for (int e = threadIdx.x; e < nvy * nvx * 3; e += kThreads) {
-        const int iyb = e / (nvx * 3), r = e - iyb * nvx * 3;  // r = ix * 3 + c
+    const float *wx = wbase + yf, *wyc = wx + xf, *wxy = wyc + gp.nvyw * Dsc;  // warp 0's tables
+    for (int e = threadIdx.x; e < nvy * nvx * 3; e += nthr) {
+        const int iyb = e / (nvx * 3), q = e - iyb * nvx * 3, v = q / 3, ch = q - v * 3;
         float s = 0.f;
-        for (int w = 0; w < kWarps; ++w) {
-            const int iw = iyb - wy_off[w];
-            if (iw >= 0 && iw < wy_n[w]) s += sm[w * wf + iw * gp.nvx * 3 + r];
+        for (int g = 0; g < gp.groups; ++g) {
+            const int iw = iyb - wy_off[g];
+            if (iw >= 0 && iw < wy_n[g]) s += wxy[(g * 3 + ch) * wf + iw * gp.nvx + v];
         }
-        oxy[iyb * gp.nvx * 3 + r] = s;
+        oxy[iyb * gp.nvx * 3 + q] = s;
     }
-    for (int e = threadIdx.x; e < 3 * nvx * Dsc; e += kThreads) {
-        const int c = e / (nvx * Dsc), r = e - c * nvx * Dsc;
+    for (int e = threadIdx.x; e < 3 * nvy * Dsc; e += nthr) {
+        const int ch = e / (nvy * Dsc), q = e - ch * nvy * Dsc, iyb = q / Dsc, j = q - iyb * Dsc;
         float s = 0.f;
-        for (int w = 0; w < kWarps; ++w) s += sm[w * wf + 3 * gp.nvyw * gp.nvx + c * gp.nvx * Dsc + r];
-        oxc[c * gp.nvx * Dsc + r] = s;
-    }
-    for (int e = threadIdx.x; e < 3 * nvy * Dsc; e += kThreads) {
-        const int c = e / (nvy * Dsc), r = e - c * nvy * Dsc, iyb = r / Dsc, j = r - iyb * Dsc;
-        float s = 0.f;
-        for (int w = 0; w < kWarps; ++w) {
-            const int iw = iyb - wy_off[w];
-            if (iw >= 0 && iw < wy_n[w])
-                s += sm[w * wf + 3 * gp.nvyw * gp.nvx + 3 * gp.nvx * Dsc + (c * gp.nvyw + iw) * Dsc + j];
+        for (int g = 0; g < gp.groups; ++g) {
+            const int iw = iyb - wy_off[g];
+            if (iw >= 0 && iw < wy_n[g]) s += wyc[(g * 3 + ch) * wf + iw * Dsc + j];
         }
-        oyc[(c * gp.nvy + iyb) * Dsc + j] = s;
+        oyc[(ch * gp.nvy + iyb) * Dsc + j] = s;
+    }
+    // X of all groups, summed into group 0's, then spread over the x vertices
+    for (int e = threadIdx.x; e < 3 * (xf / 4); e += nthr) {
+        const int ch = e / (xf / 4), i = e - ch * (xf / 4);
+        float4 *x4 = reinterpret_cast<float4 *>(wbase + ch * wf + yf) + i;
+        float4 s = *x4;
+        for (int g = 1; g < gp.groups; ++g) {
+            const float4 q = reinterpret_cast<const float4 *>(wx + (g * 3 + ch) * wf)[i];
+            s.x += q.x;
+            s.y += q.y;
+            s.z += q.z;
+            s.w += q.w;
+        }
+        *x4 = s;
+    }
+    __syncthreads();
+    for (int q = warp; q < 3 * Dsc; q += nw) {
+        const int ch = q >= Dsc ? (q >= 2 * Dsc ? 2 : 1) : 0, j = q - ch * Dsc;
+        spread_columns(wx + ch * wf + j * kTileW, cold, cs, nvx,
+                       [&](int v, float s) { oxc[(ch * gp.nvx + v) * Dsc + j] = s; });
     }
 }
 
@@ -767,10 +901,45 @@ static svdlut_status allow_dynamic_smem(const void *f, int max_optin, int device
     return SVDLUT_OK;
 }
 
+// Grid densities that the adjoint takes: 16 warps' xy, xc and yc vertices of a
+// block of BH rows within the shared memory (denser grids than about one
+// vertex per two pixels are refused).
+static bool grid_density_ok(int BH, int nvx, int H, int Dsy, int Dsc, size_t smem_limit)
+{
+    const int nvyw = span_bound((BH + kWarps - 1) / kWarps, H, Dsy);
+    const size_t warp = (3 * (static_cast<size_t>(nvyw) * nvx + static_cast<size_t>(nvx + nvyw) * Dsc) + 3) & ~size_t(3);
+    return sizeof(float) * kWarps * warp + 256 <= smem_limit;
+}
+
+// Workspace layout of a plan whose P and gp are set.
+static void layout_backward(const svdlut_dims *d, int B, BwdPlan *pl)
+{
+    const int D = d->D_t;
+    size_t off = 0;
+    pl->off_lut = off;
+    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->P * 9 * D * D);
+    pl->off_sums = off;
+    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->P * 3);
+    pl->off_grid = off;
+    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->gp.nblk * pl->gp.blk_stride);
+    pl->smax = 1;
+    for (int q = 0; q < 3; ++q) {
+        pl->sl[q] = (grid_plane_size(q, d->Dsx, d->Dsy, d->Dsc) + kGRChunk - 1) / kGRChunk;
+        pl->smax = std::max(pl->smax, pl->sl[q]);
+    }
+    pl->off_wpart = off;
+    off = align256(off + sizeof(float) * static_cast<size_t>(B) * 3 * std::max(d->K, 0) * pl->smax);
+    pl->off_prep = off;
+    pl->prep_img = prep_image_bytes(d);
+    off += static_cast<size_t>(B) * pl->prep_img;
+    pl->total = off;
+}
+
 static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit,
                                    BwdPlan *pl)
 {
     const int D = d->D_t, Dsc = d->Dsc;
+    BwdPlan best{};
     pl->lut_smem = sizeof(float) * (static_cast<size_t>(kLutWarps) * 4 * D * D + kLutWarps);
     if (pl->lut_smem > smem_limit) return fail(SVDLUT_ERR_UNSUPPORTED, "D_t=%d too large for the adjoint", D);
     // LUT pass: P CTAs per image (one CTA per SM); estimated time = waves x
@@ -789,61 +958,47 @@ static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, in
             }
         }
     }
-    // grid pass: blocks of 128 x BH; bands minimise waves x (rows a warp
-    // walks + a fixed cost of about 4 rows per block: clearing the tables,
-    // writing the partial); ties go to the better-filled waves
+    // grid pass: blocks of 128 x BH with as many row groups as fit; bands minimise
+    // waves x (rows a warp walks + a fixed cost of about 8 rows per block:
+    // clearing the tables, summing the warps, writing the partial); ties go to
+    // the better-filled waves.  Plans within svdlut_backward_noalloc's scratch
+    // go before larger ones.
     const int strips = (W + kTileW - 1) / kTileW;
     const int max_bands = std::max(1, (H + kMinBlockH - 1) / kMinBlockH);
-    int best = -1;
+    bool fits = false;
     double best_score = -1e30;
-    GridPlan bestgp{};
-    for (int bins = 1; bins >= 0 && best < 0; --bins)
     for (int bands = 1; bands <= max_bands; ++bands) {
-        GridPlan gp{};
-        gp.bins = bins;
+        BwdPlan q = *pl;
+        GridPlan &gp = q.gp;
         gp.BH = (H + bands - 1) / bands;
         gp.bands = (H + gp.BH - 1) / gp.BH;
         gp.nvx = span_bound(kTileW, W, d->Dsx);
         gp.nvy = span_bound(gp.BH, H, d->Dsy);
-        gp.rpw = (gp.BH + kWarps - 1) / kWarps;
-        gp.nvyw = span_bound(gp.rpw, H, d->Dsy);
-        const size_t need = sizeof(float) * static_cast<size_t>(kWarps) * grid_warp_floats(gp.nvx, gp.nvyw, Dsc, bins);
-        if (need + 256 > smem_limit) continue;  // + the kernel's static row offsets
+        if (!grid_density_ok(gp.BH, gp.nvx, H, d->Dsy, Dsc, smem_limit)) continue;
+        for (gp.groups = kGridGroups; gp.groups > 0; --gp.groups) {
+            gp.rpw = (gp.BH + gp.groups - 1) / gp.groups;
+            gp.nvyw = span_bound(gp.rpw, H, d->Dsy);
+            q.grid_smem = sizeof(float) * (static_cast<size_t>(grid_shared_floats(gp.nvx)) +
+                                           static_cast<size_t>(3 * gp.groups) * grid_warp_floats(gp.nvx, gp.nvyw, Dsc));
+            if (q.grid_smem + 256 <= smem_limit) break;  // + the kernel's static row offsets
+        }
+        if (gp.groups == 0) continue;
+        gp.nblk = strips * gp.bands;
+        gp.blk_stride = grid_block_floats(gp.nvx, gp.nvy, Dsc);
+        layout_backward(d, B, &q);
         const long long T = static_cast<long long>(B) * strips * gp.bands;
         const double waves = std::ceil(static_cast<double>(T) / sm_count - 1e-9);
         const double fill = static_cast<double>(T) / (waves * sm_count);
-        const double score = -waves * (gp.rpw + 4) + 1e-3 * fill;
-        if (score > best_score + 1e-12) {
+        const double score = -waves * (gp.rpw + 8) + 1e-3 * fill - (q.total > kNoAllocScratchBytes ? 1e12 : 0.0);
+        if (!fits || score > best_score + 1e-12) {
             best_score = score;
-            best = bands;
-            bestgp = gp;
+            best = q;
+            fits = true;
         }
         if (bands >= 4 * sm_count) break;
     }
-    if (best < 0) return fail(SVDLUT_ERR_UNSUPPORTED, "grid vertices too dense for the adjoint's blocks");
-    bestgp.nblk = strips * bestgp.bands;
-    bestgp.blk_stride = grid_block_floats(bestgp.nvx, bestgp.nvy, Dsc);
-    pl->gp = bestgp;
-    pl->grid_smem =
-        sizeof(float) * static_cast<size_t>(kWarps) * grid_warp_floats(bestgp.nvx, bestgp.nvyw, Dsc, bestgp.bins);
-    size_t off = 0;
-    pl->off_lut = off;
-    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->P * 9 * D * D);
-    pl->off_sums = off;
-    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->P * 3);
-    pl->off_grid = off;
-    off = align256(off + sizeof(float) * static_cast<size_t>(B) * bestgp.nblk * bestgp.blk_stride);
-    pl->smax = 1;
-    for (int q = 0; q < 3; ++q) {
-        pl->sl[q] = (grid_plane_size(q, d->Dsx, d->Dsy, Dsc) + kGRChunk - 1) / kGRChunk;
-        pl->smax = std::max(pl->smax, pl->sl[q]);
-    }
-    pl->off_wpart = off;
-    off = align256(off + sizeof(float) * static_cast<size_t>(B) * 3 * std::max(d->K, 0) * pl->smax);
-    pl->off_prep = off;
-    pl->prep_img = prep_image_bytes(d);
-    off += static_cast<size_t>(B) * pl->prep_img;
-    pl->total = off;
+    if (!fits) return fail(SVDLUT_ERR_UNSUPPORTED, "grid vertices too dense for the adjoint's blocks");
+    *pl = best;
     return SVDLUT_OK;
 }
 
@@ -977,7 +1132,7 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
         SVDLUT_CUDA_TRY(cudaGetLastError());
     }
     if (want_grid) {
-        grid_grad_kernel<<<dim3(pl.gp.nblk, B), kThreads, pl.grid_smem, s>>>(a, pl.gp, grid_part);
+        grid_grad_kernel<<<dim3(pl.gp.nblk, B), pl.gp.groups * 3 * 32, pl.grid_smem, s>>>(a, pl.gp, grid_part);
         SVDLUT_CUDA_TRY(cudaGetLastError());
         GridRed r{};
         r.B = B;

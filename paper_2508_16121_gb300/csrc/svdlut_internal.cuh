@@ -54,6 +54,9 @@ constexpr int kMaxDt = 33;
 constexpr int kMaxK = 48;
 constexpr int kMaxDsc = 64;
 
+// Scratch space of svdlut_backward_noalloc (bytes).
+constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
+
 // Validate dims against the documented ranges.
 svdlut_status check_dims(const svdlut_dims *d);
 

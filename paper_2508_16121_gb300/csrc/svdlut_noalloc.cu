@@ -15,10 +15,9 @@
 
 namespace {
 
-// Upper bound on the scratch space (bytes).  The array lives as long as the
-// library is loaded, on every GPU that loads it.
-constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
-
+// The scratch space (kNoAllocScratchBytes) lives as long as the library is
+// loaded, on every GPU that loads it.
+using svdlut::kNoAllocScratchBytes;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 // Unique id of the CUDA context current on this thread (0 if none), through
