@@ -5,10 +5,10 @@
 // forward map of Eq. 10 / Supp. Eqs. 12-22.  Passes (all on the caller's
 // stream, no atomics, every sum in a fixed order -> bitwise repeatable):
 //   1. dx      : apply_kernel<IoF32, N, true> (slopes of the same cells).
-//   2. lut     : lut_grad_kernel scatters dy * bilinear weights into
-//                warp-private tables G_p[i][j][c] (one LUT pair, all three
-//                output channels per warp: one key match per pixel and pair),
-//                then sums the warps of a CTA into a per-CTA partial.
+//   2. lut     : lut_grad_kernel adds dy * bilinear weights to warp-private
+//                tables G_p[i][j][c] (one LUT pair, all three output channels
+//                per warp), then sums the warps of a CTA into a per-CTA
+//                partial.
 //   3. grid    : grid_grad_kernel sums the folded grid planes (xy, xc, yc per
 //                output channel) over 128-px column blocks, in lane-private
 //                bins.
@@ -27,88 +27,6 @@
 
 namespace svdlut {
 
-// ---------------------------------------------------------------------------
-// deterministic warp scatter
-// ---------------------------------------------------------------------------
-
-// Position of the n-th (0-based) set bit of m (m has more than n set bits).
-__device__ __forceinline__ int nth_set_bit(unsigned int m, int n)
-{
-    int p = 0;
-#pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const unsigned int lo = p + w >= 32 ? 0xffffffffu : ((1u << (p + w)) - 1u);
-        if (__popc(m & lo) <= n) p += w;
-    }
-    return p;
-}
-
-// Adds v[corner][ch] to tab[key + off(corner) + ch], corner offsets
-// (0, ld, cs, ld + cs) for the (00, 10, 01, 11) corners of a bilinear cell.
-// Lanes with equal keys are first summed by a shuffle tree over their ranks
-// in the group (fixed order); the lowest lane of each group then writes, one
-// corner at a time with a warp barrier between corners, so two groups never
-// update one address in the same step.  key < 0 marks an inactive lane.
-// Every lane of the warp must call this.  VEC: every key's NC <= 3 values sit
-// in one 16-byte slot (tab, key, ld and cs multiples of 4 floats), updated
-// with one 16-byte load and store.
-template <int NC, bool VEC = false>
-__device__ __forceinline__ void warp_scatter(float *tab, int key, int ld, int cs, float (&v)[4][NC])
-{
-    const unsigned int full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned int me = 1u << lane;
-    const int k = key >= 0 ? key : -1 - lane;
-    const unsigned int grp = __match_any_sync(full, k);
-    if (!__all_sync(full, grp == me)) {
-        if (__all_sync(full, grp == full)) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) v[q][c] += __shfl_xor_sync(full, v[q][c], o);
-        } else {
-            const int rank = __popc(grp & (me - 1));
-            const int size = __popc(grp);
-            const int maxsize = static_cast<int>(__reduce_max_sync(full, static_cast<unsigned int>(size)));
-            for (int s = 1; s < maxsize; s <<= 1) {
-                const int src_rank = rank + s;
-                const bool take = (rank & (2 * s - 1)) == 0 && src_rank < size;
-                const int src = take ? nth_set_bit(grp, src_rank) : lane;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        const float o = __shfl_sync(full, v[q][c], src);
-                        if (take) v[q][c] += o;
-                    }
-            }
-        }
-    }
-    const bool leader = key >= 0 && (grp & (me - 1)) == 0;
-    const int off[4] = {0, ld, cs, ld + cs};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (leader) {
-            if constexpr (VEC) {
-                static_assert(NC <= 3, "one 16-byte slot per key");
-                float4 *t = reinterpret_cast<float4 *>(tab + key + off[q]);
-                float4 o = *t;
-                o.x += v[q][0];
-                if constexpr (NC > 1) o.y += v[q][1];
-                if constexpr (NC > 2) o.z += v[q][2];
-                *t = o;
-            } else {
-                float *t = tab + key + off[q];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) t[c] += v[q][c];
-            }
-        }
-        __syncwarp();
-    }
-}
-
 // Fixed-order warp sum (butterfly); every lane gets the total.
 __device__ __forceinline__ float warp_sum(float v)
 {
@@ -116,9 +34,6 @@ __device__ __forceinline__ float warp_sum(float v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-
-constexpr int kLutWarps = 12;  // 4 groups x 3 LUT pairs
-constexpr int kLutThreads = kLutWarps * 32;
 
 struct BwdArgs {
     const float *x, *dy;
@@ -133,19 +48,70 @@ struct BwdArgs {
 // LUT gradients: G^c_p[i][j] = sum_px dy_c * bilinear weight of vertex (i, j)
 // at (x_alpha, x_beta) for pair p = (alpha, beta).
 // grid (P, B); CTA (p, b) owns the rows [p H / P, (p+1) H / P) of image b.
-// Its work is the sequence of (128-column strip, row) pairs, strip by strip;
-// warp group g takes the g-th quarter of it (equal shares to within one row,
-// whatever the number of strips: a piece of a strip, whole strips, a piece of
-// the next).  Warp (group g, pair q) walks down the rows of each of its
-// pieces; lane l takes columns l + 32 k (k = 0..3: coalesced loads) and
-// keeps, per column, the four corner contributions
-// (three channels each) of its current cell in registers: while the cell
-// does not change (smooth regions, where consecutive rows fall in the same
-// cell) it only accumulates; when it changes, the warp scatters the finished
-// sums into its private table [D][D][3 channels + 1 pad] (deterministic
-// warp_scatter).  Rows are loaded two ahead.
+// Its work is the sequence of (64-column strip, row) pairs, strip by strip;
+// row group g takes the g-th share of it (equal to within one row).
+// Warp (pair q, group g) walks down the rows of its share; lane l takes
+// columns l and l + 32 and keeps, per column, the twelve corner sums (four
+// corners, three channels) of its current cell in registers: while the cell
+// does not change it only accumulates.  Finished sums wait in the warp's queue
+// (or, when most lanes finish at once, go straight on) until a batch of about
+// 32 is there: equal cells are added up (match, rank tree), then one lane per
+// cell adds its sums to the warp's own table [D][D][3], a corner at a time
+// with a warp barrier between, so two cells never update one vertex in the
+// same step.  The order of every sum is fixed: bitwise repeatable.
+// Where a run ends a few lanes at a time (smooth content: neighbouring columns
+// cross a cell border at different rows), the queue turns many nearly empty
+// batches into a full one.  Tables of three floats per vertex (13 KB) leave
+// room for 15 warps and their queues.  Noise, a new cell at every pixel, is
+// bound by the shared-memory pipe (about 85 wavefronts a batch); smooth
+// content by latency and issue slots, photos with pixel noise by the trees.
+// Measured on 8 x 1920x1080, with lut_finalize_kernel: noise 538 us, smooth
+// 287, half and half 429 (710 when each change of a lane's cell was scattered
+// at once, from 12 warps with four floats per vertex).  Also tried: one table
+// of cells (48 bytes at one place, 66 wavefronts a batch) per pair, which its
+// warps update in turns: 660, 440 and 563 us, the hand-over's latency; 12
+// warps of this kernel: 580, 323, 460 us; the queue for every batch: 671,
+// 282, 491 us.
 // Output: lut_part[b][p][c][pair][D*D], sums_part[b][p][c] (sum of dy_c).
 // ---------------------------------------------------------------------------
+constexpr int kLutGroups = 5, kLutWarps = 3 * kLutGroups;
+constexpr int kLutThreads = kLutWarps * 32;
+constexpr int kLutTileW = 64;   // columns of a strip: 32 lanes x 2
+constexpr int kLutQueue = 32;   // queued sums of a warp
+constexpr int kLutDirect = 14;  // lanes finishing at once from which the queue is passed by
+
+// floats of one warp's queue, and of one table (rounded to 4: the queues follow)
+constexpr int kLutQueueFloats = kLutQueue * 13;
+__host__ __device__ inline int lut_table_floats(int D) { return (3 * D * D + 3) & ~3; }
+__host__ __device__ inline size_t lut_grad_smem(int D)
+{
+    return sizeof(float) * (kLutWarps * (static_cast<size_t>(lut_table_floats(D)) + kLutQueueFloats) + 4 * kLutGroups);
+}
+
+// Adds the 12 sums of lanes with equal keys (key < 0: none) into the lowest
+// of them, by a tree over their ranks; returns whether this lane leads a key.
+__device__ __forceinline__ bool merge_equal_keys(int key, float (&v)[12])
+{
+    const unsigned int full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned int me = 1u << lane, lower = me - 1u;
+    const unsigned int grp = __match_any_sync(full, key >= 0 ? key : -1 - lane);
+    unsigned int g = grp;  // members that still hold a partial sum
+    while (__any_sync(full, (g & (g - 1u)) != 0u)) {
+        const unsigned int above = g & ~(me | lower);
+        const bool even = (g & me) != 0u && (__popc(g & lower) & 1) == 0;
+        const bool take = even && above != 0u;
+        const int src = take ? __ffs(above) - 1 : lane;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+            const float o = __shfl_sync(full, v[i], src);
+            if (take) v[i] += o;
+        }
+        g &= __ballot_sync(full, even);
+    }
+    return key >= 0 && (grp & lower) == 0u;
+}
+
 __global__ void __launch_bounds__(kLutThreads, 1)
     lut_grad_kernel(BwdArgs a, float *__restrict__ lut_part, float *__restrict__ sums_part)
 {
@@ -154,114 +120,182 @@ __global__ void __launch_bounds__(kLutThreads, 1)
     const int grp = warp / 3, pair = warp - grp * 3;
     const int A = pair == 2 ? 1 : 0, Bx = pair == 0 ? 1 : 2;  // axes of the pair
     const int P = gridDim.x, p = blockIdx.x, b = blockIdx.y;
-    const int D = a.D, DD = D * D;
-    float *tab = sm + warp * 4 * DD;  // [D][D][3 channels + 1 pad] of this warp's pair
-    float *sums = sm + kLutWarps * 4 * DD;
-    for (int e = threadIdx.x; e < kLutWarps * 4 * DD; e += kLutThreads) sm[e] = 0.f;
+    const int D = a.D, DD = D * D, tf = lut_table_floats(D);
+    float *tab = sm + warp * tf;  // [D][D][3] of this warp's pair
+    float4 *qv = reinterpret_cast<float4 *>(sm + kLutWarps * tf + warp * kLutQueueFloats);  // [3][kLutQueue]
+    int *qk = reinterpret_cast<int *>(qv + 3 * kLutQueue);                                   // [kLutQueue]
+    float *sums = sm + kLutWarps * (tf + kLutQueueFloats);                                   // [kLutGroups][4]
+    for (int e = threadIdx.x; e < kLutWarps * tf / 4; e += kLutThreads)
+        reinterpret_cast<float4 *>(sm)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
 
     const int r0 = static_cast<int>((static_cast<long long>(a.H) * p) / P);
     const int r1 = static_cast<int>((static_cast<long long>(a.H) * (p + 1)) / P);
-    constexpr int kGroups = kLutWarps / 3;
     const size_t plane = static_cast<size_t>(a.H) * a.W;
-    const float *xb = a.x + static_cast<size_t>(b) * 3 * plane;
+    const float *xa = a.x + (static_cast<size_t>(b) * 3 + A) * plane, *xbp = a.x + (static_cast<size_t>(b) * 3 + Bx) * plane;
     const float *gb = a.dy + static_cast<size_t>(b) * 3 * plane;
     const float fD1 = static_cast<float>(D - 1), fD2 = static_cast<float>(D - 2);
+    const int nrows = r1 - r0, strips = (a.W + kLutTileW - 1) / kLutTileW;
+    const long long T = static_cast<long long>(strips) * nrows;
+    const long long t0 = T * grp / kLutGroups, t1 = T * (grp + 1) / kLutGroups;
+    const int my_rows = static_cast<int>(t1 - t0);
+
+    float acc[2][12];  // [column][corner * 3 + channel]
+    int acc_key[2] = {-1, -1};
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int i = 0; i < 12; ++i) acc[k][i] = 0.f;
+    int qn = 0;  // queued sums
     float dysum[3] = {0.f, 0.f, 0.f};
-    float acc[4][4][3];  // [column k][corner][channel]
-    int acc_key[4] = {-1, -1, -1, -1};
+
+    // adds the sums of the lanes with key >= 0 to the table
+    auto add_batch = [&](int key, float (&v)[12]) {
+        const bool leader = merge_equal_keys(key, v);
+        const int off[4] = {0, 3 * D, 3, 3 * D + 3};
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[k][q][c] = 0.f;
-    const long long nrows = r1 - r0, T = static_cast<long long>(a.strips) * nrows;
-    const long long t1 = T * (grp + 1) / kGroups;
-    for (long long t = T * grp / kGroups; t < t1;) {
-        const int strip = static_cast<int>(t / nrows);
-        const long long s0 = strip * nrows;
-        const int ra = r0 + static_cast<int>(t - s0), rb = r0 + static_cast<int>(min(t1 - s0, nrows));
-        t = s0 + nrows;
-        const int x = strip * kTileW + lane;
-        const int n = x < a.W ? min(4, (a.W - x + 31) >> 5) : 0;  // this lane's columns x + 32 k, k < n
-        struct Row {
-            float4 pa, pb, g0, g1, g2;
-        };
-        auto load = [&](int r, Row &o) {
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            o.pa = o.pb = o.g0 = o.g1 = o.g2 = z;
-            if (r < rb && n > 0) {
-                const size_t off = static_cast<size_t>(r) * a.W + x;
-                o.pa = PixIO<float>::load_s(xb + A * plane + off, n);
-                o.pb = PixIO<float>::load_s(xb + Bx * plane + off, n);
-                o.g0 = PixIO<float>::load_s(gb + off, n);
-                o.g1 = PixIO<float>::load_s(gb + plane + off, n);
-                o.g2 = PixIO<float>::load_s(gb + 2 * plane + off, n);
+        for (int q = 0; q < 4; ++q) {
+            if (leader) {
+                float *t = tab + key * 3 + off[q];
+                const float u0 = t[0], u1 = t[1], u2 = t[2];
+                t[0] = u0 + v[q * 3];
+                t[1] = u1 + v[q * 3 + 1];
+                t[2] = u2 + v[q * 3 + 2];
             }
-        };
-        Row cur, nx1, nx2;
-        load(ra, cur);
-        load(ra + 1, nx1);
-        for (int r = ra; r < rb; ++r) {
-            load(r + 2, nx2);
+            __syncwarp();
+        }
+    };
+    auto drain = [&]() {
+        float w[12];
+        int k = -1;
+        __syncwarp();
+        if (lane < qn) {
+            const float4 q0 = qv[lane], q1 = qv[kLutQueue + lane], q2 = qv[2 * kLutQueue + lane];
+            w[0] = q0.x;
+            w[1] = q0.y;
+            w[2] = q0.z;
+            w[3] = q0.w;
+            w[4] = q1.x;
+            w[5] = q1.y;
+            w[6] = q1.z;
+            w[7] = q1.w;
+            w[8] = q2.x;
+            w[9] = q2.y;
+            w[10] = q2.z;
+            w[11] = q2.w;
+            k = qk[lane];
+        } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const bool act = k < n;
-                const float gy[3] = {get(cur.g0, k), get(cur.g1, k), get(cur.g2, k)};
+            for (int i = 0; i < 12; ++i) w[i] = 0.f;
+        }
+        qn = 0;
+        add_batch(k, w);
+    };
+    // the sums v of the lanes with key >= 0 are finished
+    auto finish = [&](int key, float (&v)[12]) {
+        const unsigned int done = __ballot_sync(0xffffffffu, key >= 0);
+        const int cnt = __popc(done);
+        if (cnt >= kLutDirect) {
+            add_batch(key, v);
+            return;
+        }
+        if (qn + cnt > kLutQueue) drain();
+        if (key >= 0) {
+            const int s = qn + __popc(done & ((1u << lane) - 1u));
+            qv[s] = make_float4(v[0], v[1], v[2], v[3]);
+            qv[kLutQueue + s] = make_float4(v[4], v[5], v[6], v[7]);
+            qv[2 * kLutQueue + s] = make_float4(v[8], v[9], v[10], v[11]);
+            qk[s] = key;
+        }
+        qn += cnt;
+    };
+
+    struct Row {
+        float pa[2], pb[2], g[3][2];
+        int n;  // this lane's columns: 0, 1 or 2
+    };
+    // rows are loaded one ahead of their use, from the cursor (strip, row)
+    int ls = static_cast<int>(t0 / nrows), lr = static_cast<int>(t0 - ls * static_cast<long long>(nrows)), loaded = 0;
+    auto load = [&](Row &o) {
+        const int x = ls * kLutTileW + lane;
+        o.n = loaded < my_rows ? (x < a.W) + (x + 32 < a.W) : 0;
+        const size_t off = static_cast<size_t>(r0 + lr) * a.W + x;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) dysum[c] += gy[c];
-                float da, db;
-                const int ia = cell_of(fminf(fmaxf(get(cur.pa, k), 0.f), 1.f), fD1, fD2, da);
-                const int ib = cell_of(fminf(fmaxf(get(cur.pb, k), 0.f), 1.f), fD1, fD2, db);
-                const float w[4] = {(1.f - da) * (1.f - db), da * (1.f - db), (1.f - da) * db, da * db};
-                const int key = act ? (ia * D + ib) * 4 : -1;
-                const bool change = key != acc_key[k];
-                if (__any_sync(0xffffffffu, change))
-                    warp_scatter<3, true>(tab, change ? acc_key[k] : -1, D * 4, 4, acc[k]);
-                if (change) {
+        for (int k = 0; k < 2; ++k) {
+            const bool in = k < o.n;
+            o.pa[k] = in ? __ldcs(xa + off + 32 * k) : 0.f;
+            o.pb[k] = in ? __ldcs(xbp + off + 32 * k) : 0.f;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
+            for (int c = 0; c < 3; ++c) o.g[c][k] = in ? __ldcs(gb + c * plane + off + 32 * k) : 0.f;
+        }
+        ++loaded;
+        if (++lr == nrows) {
+            lr = 0;
+            ++ls;
+        }
+    };
+    Row cur, nxt;
+    load(cur);
+    for (int r = 0; r < my_rows; ++r) {
+        load(nxt);
+        float da[2], db[2];
+        int key[2];
+        bool change[2];
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) acc[k][q][c] = gy[c] * w[q];
-                    acc_key[k] = key;
-                } else {
+        for (int k = 0; k < 2; ++k) {
+            const int ia = cell_of(__saturatef(cur.pa[k]), fD1, fD2, da[k]);
+            const int ib = cell_of(__saturatef(cur.pb[k]), fD1, fD2, db[k]);
+            key[k] = ia * D + ib;
+            change[k] = k < cur.n && key[k] != acc_key[k];
+        }
+        if (__any_sync(0xffffffffu, change[0] || change[1])) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
+            for (int k = 0; k < 2; ++k) {
+                finish(change[k] ? acc_key[k] : -1, acc[k]);
+                if (change[k]) {
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) acc[k][q][c] = fmaf(gy[c], w[q], acc[k][q][c]);
+                    for (int i = 0; i < 12; ++i) acc[k][i] = 0.f;
+                    acc_key[k] = key[k];
                 }
             }
-            cur = nx1;
-            nx1 = nx2;
         }
-        // the piece's runs end here
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            warp_scatter<3, true>(tab, acc_key[k], D * 4, 4, acc[k]);
-            acc_key[k] = -1;
+        for (int k = 0; k < 2; ++k) {
+            const float w[4] = {(1.f - da[k]) * (1.f - db[k]), da[k] * (1.f - db[k]), (1.f - da[k]) * db[k], da[k] * db[k]};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                dysum[c] += cur.g[c][k];
+                // a column outside the image adds nothing (its dy is 0)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[k][q * 3 + c] = fmaf(cur.g[c][k], w[q], acc[k][q * 3 + c]);
+            }
         }
+        cur = nxt;
     }
+    finish(acc_key[0], acc[0]);
+    finish(acc_key[1], acc[1]);
+    drain();
+
     // sum of dy_c: the pair-0 warps' totals (every pair warp of a group sees the same pixels)
 #pragma unroll
     for (int c = 0; c < 3; ++c) dysum[c] = warp_sum(dysum[c]);
     if (lane == 0 && pair == 0) {
-        sums[grp * 3 + 0] = dysum[0];
-        sums[grp * 3 + 1] = dysum[1];
-        sums[grp * 3 + 2] = dysum[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sums[grp * 4 + c] = dysum[c];
     }
     __syncthreads();
-    // CTA partial [c][pair][cell]: sum the groups in order
+    // CTA partial [c][pair][vertex]: sum the groups in order
     float *out = lut_part + (static_cast<size_t>(b) * P + p) * 9 * DD;
     for (int e = threadIdx.x; e < 9 * DD; e += kLutThreads) {
-        const int c = e / (3 * DD), r = e - c * 3 * DD, q = r / DD, cell = r - q * DD;
+        const int c = e / (3 * DD), r = e - c * 3 * DD, q = r / DD, vtx = r - q * DD;
         float s = 0.f;
-        for (int gq = 0; gq < kGroups; ++gq) s += sm[(gq * 3 + q) * 4 * DD + cell * 4 + c];
+#pragma unroll
+        for (int g = 0; g < kLutGroups; ++g) s += sm[(g * 3 + q) * tf + vtx * 3 + c];
         out[e] = s;
     }
     if (threadIdx.x < 3) {
         float s = 0.f;
-        for (int gq = 0; gq < kGroups; ++gq) s += sums[gq * 3 + threadIdx.x];
+        for (int g = 0; g < kLutGroups; ++g) s += sums[g * 4 + threadIdx.x];
         sums_part[(static_cast<size_t>(b) * P + p) * 3 + threadIdx.x] = s;
     }
 }
@@ -935,36 +969,40 @@ static void layout_backward(const svdlut_dims *d, int B, BwdPlan *pl)
     pl->total = off;
 }
 
-static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit,
-                                   BwdPlan *pl)
+// LUT pass: CTAs per image, at most max_p (one CTA per SM); estimated time =
+// waves x (rows a group walks: its share of strips x rows, + a fixed cost of
+// about 16 rows per CTA: clearing the tables, writing the partial) + a row's
+// time per 24 partials that lut_finalize_kernel sums.
+static int plan_lut_ctas(int B, int H, int W, int sm_count, int max_p)
 {
-    const int D = d->D_t, Dsc = d->Dsc;
-    BwdPlan best{};
-    pl->lut_smem = sizeof(float) * (static_cast<size_t>(kLutWarps) * 4 * D * D + kLutWarps);
-    if (pl->lut_smem > smem_limit) return fail(SVDLUT_ERR_UNSUPPORTED, "D_t=%d too large for the adjoint", D);
-    // LUT pass: P CTAs per image (one CTA per SM); estimated time = waves x
-    // (rows a warp group walks: a quarter of strips x rows, + a fixed cost of
-    // about 16 rows per CTA: clearing the tables, writing the partial)
-    {
-        const long long strips = (W + kTileW - 1) / kTileW, G = kLutWarps / 3;
-        long long best_cost = -1;
-        for (int P = 1; P <= std::min(H, 4 * sm_count); ++P) {
-            const long long waves = (static_cast<long long>(B) * P + sm_count - 1) / sm_count;
-            const long long rows = (H + P - 1) / P;
-            const long long cost = waves * ((strips * rows + G - 1) / G + 16);
-            if (best_cost < 0 || cost < best_cost) {
-                best_cost = cost;
-                pl->P = P;
-            }
+    const long long strips = (W + kLutTileW - 1) / kLutTileW;
+    long long best_cost = -1;
+    int best = 1;
+    for (int P = 1; P <= std::min({H, 4 * sm_count, max_p}); ++P) {
+        const long long waves = (static_cast<long long>(B) * P + sm_count - 1) / sm_count;
+        const long long rows = (H + P - 1) / P;
+        const long long cost = 24 * waves * ((strips * rows + kLutGroups - 1) / kLutGroups + 16) + P;
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = P;
         }
     }
-    // grid pass: blocks of 128 x BH with as many row groups as fit; bands minimise
-    // waves x (rows a warp walks + a fixed cost of about 8 rows per block:
-    // clearing the tables, summing the warps, writing the partial); ties go to
-    // the better-filled waves.  Plans within svdlut_backward_noalloc's scratch
-    // go before larger ones.
+    return best;
+}
+
+// Grid pass of a plan whose P is set: blocks of 128 x BH with as many row
+// groups as fit; bands minimise waves x (rows a warp walks + a fixed cost of
+// about 8 rows per block: clearing the tables, summing the warps, writing the
+// partial), ties go to the better-filled waves, and plans within
+// svdlut_backward_noalloc's scratch go before larger ones.  smallest: the
+// smallest workspace instead.  False if no block fits.
+static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit, bool smallest,
+                      BwdPlan *pl)
+{
+    const int Dsc = d->Dsc;
     const int strips = (W + kTileW - 1) / kTileW;
     const int max_bands = std::max(1, (H + kMinBlockH - 1) / kMinBlockH);
+    BwdPlan best{};
     bool fits = false;
     double best_score = -1e30;
     for (int bands = 1; bands <= max_bands; ++bands) {
@@ -989,7 +1027,8 @@ static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, in
         const long long T = static_cast<long long>(B) * strips * gp.bands;
         const double waves = std::ceil(static_cast<double>(T) / sm_count - 1e-9);
         const double fill = static_cast<double>(T) / (waves * sm_count);
-        const double score = -waves * (gp.rpw + 8) + 1e-3 * fill - (q.total > kNoAllocScratchBytes ? 1e12 : 0.0);
+        const double score = smallest ? -static_cast<double>(q.total)
+                                      : -waves * (gp.rpw + 8) + 1e-3 * fill - (q.total > kNoAllocScratchBytes ? 1e12 : 0.0);
         if (!fits || score > best_score + 1e-12) {
             best_score = score;
             best = q;
@@ -997,8 +1036,37 @@ static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, in
         }
         if (bands >= 4 * sm_count) break;
     }
-    if (!fits) return fail(SVDLUT_ERR_UNSUPPORTED, "grid vertices too dense for the adjoint's blocks");
-    *pl = best;
+    if (fits) *pl = best;
+    return fits;
+}
+
+static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit,
+                                   BwdPlan *pl)
+{
+    pl->lut_smem = lut_grad_smem(d->D_t);
+    if (pl->lut_smem > smem_limit) return fail(SVDLUT_ERR_UNSUPPORTED, "D_t=%d too large for the adjoint", d->D_t);
+    pl->P = plan_lut_ctas(B, H, W, sm_count, H);
+    if (!plan_grid(d, B, H, W, sm_count, smem_limit, false, pl))
+        return fail(SVDLUT_ERR_UNSUPPORTED, "grid vertices too dense for the adjoint's blocks");
+    if (pl->total > kNoAllocScratchBytes) {
+        // stay within svdlut_backward_noalloc's scratch where fewer LUT CTAs
+        // and the smallest grid plan do
+        BwdPlan q = *pl;
+        q.P = 1;
+        plan_grid(d, B, H, W, sm_count, smem_limit, true, &q);
+        if (q.total <= kNoAllocScratchBytes) {
+            const size_t per = sizeof(float) * static_cast<size_t>(B) * (9 * d->D_t * d->D_t + 3);
+            q.P = std::min(pl->P, static_cast<int>(1 + (kNoAllocScratchBytes - q.total) / per));
+            layout_backward(d, B, &q);
+            while (q.total > kNoAllocScratchBytes) {  // the parts' alignment
+                --q.P;
+                layout_backward(d, B, &q);
+            }
+            q.P = plan_lut_ctas(B, H, W, sm_count, q.P);
+            plan_grid(d, B, H, W, sm_count, smem_limit, false, &q);
+            *pl = q;
+        }
+    }
     return SVDLUT_OK;
 }
 

@@ -42,3 +42,36 @@ def test_grid_gradients_at_tile_edges(H, W, Dsx, Dsy, Dsc):
     d = si.Dims(9, 3, 5, Dsx, Dsy, Dsc)
     x, p = si.make_batch(700 + H + W, 2, H, W, d)
     check(x, p, si.make_upstream(701 + H, x.shape), d)
+
+
+# (H, W, D_t, image): 64-column strips with 1, 63, 64 and 65 columns, shares
+# without rows, one LUT cell and the largest table; every lane in one cell,
+# every lane in its own, a few cells per warp, and runs that end a few lanes at
+# a time (the queue)
+@pytest.mark.parametrize("H,W,D,mode", [
+    (1, 1, 2, "noise"), (2, 63, 33, "noise"), (5, 64, 33, "constant"), (3, 65, 17, "smooth"), (40, 130, 33, "noise"),
+    (70, 97, 33, "dither"), (64, 64, 2, "noise"), (37, 200, 33, "smooth")])
+def test_lut_gradients_at_strip_and_queue_edges(H, W, D, mode):
+    d = si.Dims(D, min(D, 8), 3, 2, 2, 5)
+    x, p = si.make_batch(720 + H + W, 2, H, W, d, mode=mode if mode in ("noise", "smooth") else "smooth")
+    if mode == "constant":
+        x[...] = np.float32(0.3125 + 1 / 64)
+    if mode == "dither":  # flat areas whose pixels fall in a few neighbouring cells
+        x = np.clip(0.4 + np.random.default_rng(722).normal(0, 0.02, x.shape), 0, 1).astype(np.float32)
+    dy = si.make_upstream(721 + H, x.shape)
+    check(x, p, dy, d)
+
+
+def test_lut_gradients_are_bitwise_repeatable():
+    import torch
+    import paper_2508_16121_gb300 as sv
+    H, W = 150, 333
+    d = si.spatial_dims(H, W)
+    x, p = si.make_batch(740, 2, H, W, d)
+    xt, pt = torch.from_numpy(x).cuda(), sv.to_device(p)
+    dy = torch.from_numpy(si.make_upstream(741, x.shape)).cuda()
+    first = sv.backward(xt, pt, dy)
+    for _ in range(3):
+        again = sv.backward(xt, pt, dy)
+        for k in first:
+            assert torch.equal(first[k], again[k]), k
