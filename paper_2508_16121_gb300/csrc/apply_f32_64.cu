@@ -1,0 +1,5 @@
+// apply_kernel for the transform of float images, up to 64 per launch.
+#include "apply_instances.cuh"
+
+template svdlut_status svdlut::launch_io<svdlut::IoF32, 64, false>(svdlut::LaunchArgs<64> &, size_t,
+                                                            const svdlut::DeviceInfo &, cudaStream_t, int);

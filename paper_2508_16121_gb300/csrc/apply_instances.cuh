@@ -1,0 +1,37 @@
+// The instances of apply_kernel: included by the translation units that
+// instantiate launch_io, one (format, N, direction) each, so that they compile
+// in parallel and once.
+#pragma once
+
+#include "apply_kernel.cuh"
+#include "apply_launch.cuh"
+
+namespace svdlut {
+
+// Launches one instance as a dependent of the preceding kernel (prep_kernel, or
+// any other): it may be launched while that one runs, and waits for it before
+// it reads anything (with PRE, before it reads the tables: prep_kernel has
+// waited for what came before).
+template <class IO, int N, bool DX, bool PRE, bool FAST>
+svdlut_status launch_instance(LaunchArgs<N> &a, size_t smem, const DeviceInfo &di, cudaStream_t s, int grid)
+{
+    svdlut_status st = allow_smem_once(reinterpret_cast<const void *>(apply_kernel<IO, N, DX, PRE, FAST>),
+                                       di.max_smem_optin, di.device);
+    if (st != SVDLUT_OK) return st;
+    if ((st = check_buffer(&a.check)) != SVDLUT_OK) return st;
+    if (grid <= 0) grid = std::min(a.total_blocks, di.sm_count);
+    grid = std::max(1, std::min(grid, a.total_blocks));
+    return launch_pdl(apply_kernel<IO, N, DX, PRE, FAST>, dim3(grid), dim3(kThreads), smem, s, a);
+}
+
+template <class IO, int N, bool DX>
+svdlut_status launch_io(LaunchArgs<N> &a, size_t smem, const DeviceInfo &di, cudaStream_t s, int grid)
+{
+    if (a.pre) return launch_instance<IO, N, DX, true, false>(a, smem, di, s, grid);
+    bool fast = a.xcol != 0;
+    for (int i = 0; i < a.n; ++i) fast = fast && fast_rows(a.img[i]);
+    return fast ? launch_instance<IO, N, DX, false, true>(a, smem, di, s, grid)
+                : launch_instance<IO, N, DX, false, false>(a, smem, di, s, grid);
+}
+
+}  // namespace svdlut

@@ -71,7 +71,7 @@ struct LaunchArgs {
     int lcell_floats;    // floats reserved for the cell table
     int scratch_floats;  // floats of the block buffers / prologue temporaries
     int xcol;            // nonzero: per-column xc tables (every image's Dsc <= kXcolMaxDsc)
-    int pre;             // nonzero: cell tables and folded grids precomputed (ImgDesc::pcell, pfold)
+    int pre;             // nonzero: cell tables and folded grids precomputed (the PRE kernel)
     unsigned int *queue;  // non-null: blocks are taken from this counter (must be 0 at launch)
     unsigned int *check;  // index-check status (builds with SVDLUT_CHECK_BOUNDS), else null
     ImgDesc img[N];
@@ -522,7 +522,7 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-__device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+__host__ __device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 __device__ inline void build_luts(const ImgDesc &d, float4 *lcell, float *tmp, float *misc, int tmp_floats,
                                   unsigned int *check)
@@ -537,9 +537,7 @@ __device__ inline void build_luts(const ImgDesc &d, float4 *lcell, float *tmp, f
     float *sV = tmp + nf * DRp;        // [nf][D][Rp]
     float4 *vt = reinterpret_cast<float4 *>(tmp + 2 * nf * DRp);  // [D][D]
 
-    // grid weights and summed biases
-    for (int e = tid; e < d.K * 4; e += kThreads) misc[e] = __ldg(d.gw + e);
-    if (tid < 3) {
+    if (tid < 3) {  // summed biases
         float b = __ldg(d.lw + tid * 4 + 3);
         for (int k = tid; k < d.K; k += 3) b += __ldg(d.gw + k * 4 + 3);
         misc[kMaxK * 4 + tid] = b;
@@ -657,6 +655,106 @@ __device__ inline void build_luts(const ImgDesc &d, float4 *lcell, float *tmp, f
     }
 }
 
+// ---- the same tables for rank 8, overlapped with the grid fold ----
+// build_luts is a chain of phases (factors, products of one pair, its cells,
+// the next pair).  For the paper's rank the factors arrive by
+// asynchronous copies into the part of the block buffers that is not in use
+// yet (the xc slice and the row tables) while the block's grids are folded,
+// and one pass builds the cells from them: a thread holds the U rows i and
+// i + 1 of a pair's three tables and walks along j, one V row a step, the
+// products in the order of build_luts (the same bits).
+constexpr int kFastRank = 8, kFastRp = 12;  // rank, row stride in floats (as padded_rank)
+__host__ __device__ inline int fast_factor_floats(int D) { return 2 * 9 * D * kFastRp + 9 * kFastRank + 12; }
+
+__host__ __device__ __forceinline__ bool fast_factors_ok(const ImgDesc &d)
+{
+    return d.R == kFastRank && aligned16(d.U) && aligned16(d.V) && aligned16(d.S) && aligned16(d.lw);
+}
+
+// Issues the copies of image d's factors to buf: U, V [9][D][kFastRp], S
+// [9][8], lut_w [3][4]; and the summed biases.
+__device__ inline void copy_factors(const ImgDesc &d, float *buf, float *misc)
+{
+    const int tid = threadIdx.x, nrow = 9 * d.D, half = nrow * kFastRp;
+    for (int e = tid; e < nrow * 2; e += kThreads) {  // 16-byte chunks of the rows
+        const int row = e >> 1, q = 4 * (e & 1);
+        cp_async16(buf + row * kFastRp + q, d.U + row * kFastRank + q);
+        cp_async16(buf + half + row * kFastRp + q, d.V + row * kFastRank + q);
+    }
+    if (tid < 18) cp_async16(buf + 2 * half + 4 * tid, d.S + 4 * tid);
+    else if (tid < 21) cp_async16(buf + 2 * half + 4 * tid, d.lw + 4 * (tid - 18));
+    else if (tid >= 32 && tid < 35) {
+        const int c = tid - 32;
+        float b = __ldg(d.lw + c * 4 + 3);
+        for (int k = c; k < d.K; k += 3) b += __ldg(d.gw + k * 4 + 3);
+        misc[kMaxK * 4 + c] = b;
+    }
+}
+
+__device__ __forceinline__ float dot8(const float (&u)[8], const float4 &v0, const float4 &v1)
+{
+    const float a = fmaf(u[0], v0.x, fmaf(u[1], v0.y, fmaf(u[2], v0.z, u[3] * v0.w)));
+    return fmaf(u[4], v1.x, fmaf(u[5], v1.y, fmaf(u[6], v1.z, fmaf(u[7], v1.w, a))));
+}
+
+// The cell table from the factors in buf (copies complete, visible to all).
+__device__ inline void build_cells(int D, const float *buf, float4 *lcell)
+{
+    const int Dm1 = D - 1, DRp = D * kFastRp, half = 9 * DRp;
+    const float *sS = buf + 2 * half, *sW = sS + 9 * kFastRank;
+    const int rows = 3 * Dm1, nseg = max(1, min(Dm1, kThreads / rows));
+    for (int e = threadIdx.x; e < nseg * rows; e += kThreads) {
+        const int seg = e / rows, rem = e - seg * rows, p = rem / Dm1, i = rem - p * Dm1;
+        const int j0 = Dm1 * seg / nseg, j1 = Dm1 * (seg + 1) / nseg;
+        float u0[3][8], u1[3][8];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float *u = buf + (c * 3 + p) * DRp + i * kFastRp, *sc = sS + (c * 3 + p) * kFastRank;
+            const float w = sW[c * 4 + p];
+#pragma unroll
+            for (int q = 0; q < 8; q += 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(u + q);
+                const float4 b = *reinterpret_cast<const float4 *>(u + kFastRp + q);
+                const float4 s = *reinterpret_cast<const float4 *>(sc + q);
+                u0[c][q] = a.x * s.x * w, u0[c][q + 1] = a.y * s.y * w, u0[c][q + 2] = a.z * s.z * w,
+                u0[c][q + 3] = a.w * s.w * w;
+                u1[c][q] = b.x * s.x * w, u1[c][q + 1] = b.y * s.y * w, u1[c][q + 2] = b.z * s.z * w,
+                u1[c][q + 3] = b.w * s.w * w;
+            }
+        }
+        float t0[3], t1[3];  // T(i, j), T(i + 1, j) of the three channels
+        auto column = [&](int j, float (&a)[3], float (&b)[3]) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float4 *v = reinterpret_cast<const float4 *>(buf + half + (c * 3 + p) * DRp + j * kFastRp);
+                const float4 v0 = v[0], v1 = v[1];
+                a[c] = dot8(u0[c], v0, v1);
+                b[c] = dot8(u1[c], v0, v1);
+            }
+        };
+        column(j0, t0, t1);
+        float4 *q = lcell + (p * Dm1 * D + i * D + j0) * 3;
+        for (int j = j0; j < j1; ++j, q += 3) {
+            float n0[3], n1[3], bb[3], cc[3], dd[3];
+            column(j + 1, n0, n1);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                bb[c] = t1[c] - t0[c];
+                cc[c] = n0[c] - t0[c];
+                dd[c] = n1[c] - t1[c] - n0[c] + t0[c];
+            }
+            q[0] = make_float4(t0[0], t0[1], t0[2], bb[0]);
+            q[1] = make_float4(bb[1], bb[2], cc[0], cc[1]);
+            q[2] = make_float4(cc[2], dd[0], dd[1], dd[2]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                t0[c] = n0[c];
+                t1[c] = n1[c];
+            }
+        }
+    }
+}
+
 struct BlockGeom {
     int x0, y0, rows, ixlo, iylo, nvx, nvy;
 };
@@ -750,8 +848,8 @@ __device__ __forceinline__ BlockBufs block_bufs(float *scratch, int nvx, int nvy
 // Block setup, phase A: grid slices of the block footprint folded per output
 // channel (sum over grids k = c mod 3 of w_k times grid k: Supp. Eqs. 21-22);
 // column and row cell tables.
-__device__ inline void block_phase_a(const ImgDesc &d, const BlockGeom &g, const BlockBufs &b, const float *misc,
-                                     bool fold = true)
+template <bool FOLD>
+__device__ inline void block_phase_a(const ImgDesc &d, const BlockGeom &g, const BlockBufs &b)
 {
     const int tid = threadIdx.x;
     const int nvx = g.nvx, nvy = g.nvy, Dsc = d.Dsc, K = d.K;
@@ -762,7 +860,7 @@ __device__ inline void block_phase_a(const ImgDesc &d, const BlockGeom &g, const
     // thread takes kFoldBatch elements at a time and issues all their loads
     // before the first FMA, so the slices cost a few memory round trips.
     const int nxy = 3 * nvy * nvx, nxc = 3 * nvx * Dsc, nyc = 3 * nvy * Dsc, ntot = nxy + nxc + nyc;
-    if (!fold) {
+    if constexpr (!FOLD) {
         // the folded slices were copied from the precomputed ones (setup_pre)
     } else if (K > 0) {
         // element e -> its first grid value's address and its channel c (by
@@ -813,13 +911,14 @@ __device__ inline void block_phase_a(const ImgDesc &d, const BlockGeom &g, const
 #pragma unroll
                 for (int t = 0; t < kFoldTerms; ++t) {
                     const int k = ch[q] + 3 * t;
-                    if (k < K) acc = fmaf(misc[k * 4 + which], v[q][t], acc);
+                    if (k < K) acc = fmaf(__ldg(d.gw + k * 4 + which), v[q][t], acc);
                 }
                 if (K > 3 * kFoldTerms) {  // grids beyond the third of a channel
                     int c;
                     size_t kst;
                     const float *sp = locate(e, c, kst);
-                    for (int k = c + 3 * kFoldTerms; k < K; k += 3) acc = fmaf(misc[k * 4 + which], __ldg(sp + k * kst), acc);
+                    for (int k = c + 3 * kFoldTerms; k < K; k += 3)
+                        acc = fmaf(__ldg(d.gw + k * 4 + which), __ldg(sp + k * kst), acc);
                 }
                 float *dst = e < nxy ? b.fxy + e : (e < nxy + nxc ? b.fxc + (e - nxy) : b.fyc + (e - nxy - nxc));
                 *dst = acc;
@@ -1180,6 +1279,15 @@ __device__ __forceinline__ const float4 *lut_at(const float4 *lcell, unsigned in
 #endif
 }
 
+// Fast rows (the common case, uniform over a block): per-column xc tables,
+// D - 1 = 2 (Dsc - 1) (the slice cell is the LUT cell halved: the 17 intensity
+// vertices are every other LUT vertex), and x-cells at least 3 pixels wide (a
+// lane's 4 pixels touch at most 2 of them).
+__host__ __device__ __forceinline__ bool fast_rows(const ImgDesc &d)
+{
+    return d.D - 1 == 2 * (d.Dsc - 1) && d.W - 1 >= 3 * (d.Dsx - 1);
+}
+
 // DX = false: the forward transform, y = f(x).
 // DX = true (float images): the pixel part of the adjoint, dx = (df/dx)^T dy,
 // from the slopes of the same cell coefficients (lut_pair_dx); the xc / yc
@@ -1190,7 +1298,13 @@ __device__ __forceinline__ const float4 *lut_at(const float4 *lcell, unsigned in
 // plane).  Every pixel gathers its own cells: reusing a lane's previous cell
 // when unchanged saved shared-memory wavefronts in smooth regions but cost
 // more in compares than it saved.
-template <class IO, int N, bool DX>
+// PRE: cell tables and folded grids come from prep_kernel (ImgDesc::pcell,
+// pfold); otherwise every CTA builds them.  FAST: every image takes fast rows;
+// otherwise each block decides.  Both are template parameters because the
+// pixel loop needs all 128 registers: with the table construction and the
+// general rows in the same kernel it spilled, and 4K frames took 100 us
+// instead of 94 (PRE alone is small enough for both kinds of rows).
+template <class IO, int N, bool DX, bool PRE, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constant__ LaunchArgs<N> a)
 {
     extern __shared__ __align__(16) float smem[];
@@ -1201,8 +1315,9 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
     // the next kernel of the stream (e.g. the next call's prep_kernel, which
     // waits for this one before reading anything) may begin launching
     asm volatile("griddepcontrol.launch_dependents;\n" :::);
+    if constexpr (!PRE) asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool xcol = a.xcol != 0;
+    const bool xcol = FAST || a.xcol != 0;
     // Block schedule: a contiguous range per CTA, or (queue) blocks taken in
     // order from a global counter so that uneven blocks balance out.
     int *slot = reinterpret_cast<int *>(misc + kMaxK * 4 + 3);
@@ -1266,7 +1381,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
 
     Raw cur[NP], nxt[NP];
     int cur_im = -1;
-    bool first = true, pre_wait = a.pre != 0;
+    bool first = true, pre_wait = PRE;
     for (;;) {
         const int im = find_image(blk);
         const ImgDesc &d = a.img[im];
@@ -1281,7 +1396,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
             }
         };
         __syncthreads();  // previous block's rows done with the buffers and the cell table
-        if (a.pre) {
+        if constexpr (PRE) {
             // The pixels are inputs of the call, complete before the launch:
             // the first row is requested while the precomputation may still
             // run (programmatic dependent launch); the tables after it ends.
@@ -1293,14 +1408,29 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
             setup_pre(d, g, b, lcell, misc, im != cur_im);
             cp_async_wait_all();
             __syncthreads();
-        } else if (im != cur_im) {
-            build_luts(d, lcell, scratch, misc, a.scratch_floats, a.check);
-            __syncthreads();
+        }
+        // the factors' place: the block buffers from the xc slice on
+        const bool overlap = !PRE && im != cur_im && fast_factors_ok(d) &&
+                             (b.xcol - scratch) + fast_factor_floats(d.D) <= a.scratch_floats;
+        if constexpr (!PRE) {
+            if (overlap) {
+                copy_factors(d, b.xcol, misc);
+            } else if (im != cur_im) {
+                build_luts(d, lcell, scratch, misc, a.scratch_floats, a.check);
+                __syncthreads();
+            }
         }
         cur_im = im;
         first_row();
         if (a.queue && threadIdx.x == 0) *slot = static_cast<int>(atomicAdd(a.queue, 1u));
-        block_phase_a(d, g, b, misc, !a.pre);
+        block_phase_a<!PRE>(d, g, b);
+        if constexpr (!PRE) {
+            if (overlap) {
+                cp_async_wait_all();
+                __syncthreads();
+                build_cells(d.D, b.xcol, lcell);
+            }
+        }
         __syncthreads();
         const int next = a.queue ? *slot : blk + 1;
         const bool has_next = next < b_end;
@@ -1345,16 +1475,11 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                 sl = fmaf(q.w, dxk[k], q.y);
             }
         };
-        // Fast rows (the common case, uniform over the block): per-column xc
-        // tables, D - 1 = 2 (Dsc - 1) (the slice cell is the LUT cell halved:
-        // the 17 intensity vertices are every other LUT vertex), and x-cells
-        // at least 3 pixels wide (a lane's 4 pixels touch at most 2 of them).
-        const bool fast = xcol && D - 1 == 2 * Dc1 && d.W - 1 >= 3 * (d.Dsx - 1);
         auto rows = [&](auto fast_tag) {
-            constexpr bool FAST = decltype(fast_tag)::value;
+            constexpr bool FAST_ROWS = decltype(fast_tag)::value;
             // fast rows: xy of pixel k = xa + w0[k] (xb - xa) + w1[k] (xc - xb)
             float w0[4], w1[4];
-            if constexpr (FAST) {
+            if constexpr (FAST_ROWS) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const bool c0 = ixl[k] == ixl[0];
@@ -1373,7 +1498,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                 warp_row_tables(g, b, Dsc, row);
                 __syncwarp();
                 float out[3][4];
-                if constexpr (FAST) {
+                if constexpr (FAST_ROWS) {
                     const float4 xa = b.rxy[ixl[0]], xb = b.rxy[ixl[0] + 1], xc = b.rxy[min(ixl[0] + 2, g.nvx - 1)];
                     const float base[3] = {bias0 + xa.x, bias1 + xa.y, bias2 + xa.z};
                     const float ab[3] = {xb.x - xa.x, xb.y - xa.y, xb.z - xa.z};
@@ -1533,8 +1658,12 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                 for (int c = 0; c < NP; ++c) cur[c] = nxt[c];
             }
         };
-        if (fast) rows(std::true_type{});
-        else rows(std::false_type{});
+        if constexpr (FAST) {
+            rows(std::true_type{});
+        } else {
+            if (xcol && fast_rows(d)) rows(std::true_type{});
+            else rows(std::false_type{});
+        }
         if (warp >= g.rows && has_next) load_row(next, warp, cur);  // no row here
         if (!has_next) break;
         blk = next;

@@ -115,24 +115,10 @@ inline svdlut_status allow_smem_once(const void *fn, int max_smem, int device)
     return SVDLUT_OK;
 }
 
+// Launches apply_kernel<IO, N, DX, ..> for args whose blocks are planned
+// (instances in apply_instances.cuh's translation units).
 template <class IO, int N, bool DX>
-svdlut_status launch_apply_t(LaunchArgs<N> &a, size_t smem, int sm_count, int max_smem, int device,
-                             cudaStream_t s, int grid)
-{
-    svdlut_status st = allow_smem_once(reinterpret_cast<const void *>(apply_kernel<IO, N, DX>), max_smem, device);
-    if (st != SVDLUT_OK) return st;
-    if ((st = check_buffer(&a.check)) != SVDLUT_OK) return st;
-    if (grid <= 0) grid = std::min(a.total_blocks, sm_count);
-    grid = std::max(1, std::min(grid, a.total_blocks));
-    if (a.pre) {
-        // dependent of the preceding prep_kernel: it may start while that
-        // kernel runs and waits for it before reading the tables
-        return launch_pdl(apply_kernel<IO, N, DX>, dim3(grid), dim3(kThreads), smem, s, a);
-    }
-    apply_kernel<IO, N, DX><<<grid, kThreads, smem, s>>>(a);
-    SVDLUT_CUDA_TRY(cudaGetLastError());
-    return SVDLUT_OK;
-}
+svdlut_status launch_io(LaunchArgs<N> &a, size_t smem, const DeviceInfo &di, cudaStream_t s, int grid);
 
 // Workspace bytes of the precomputed tables of one image, and the launch of
 // prep_kernel over a chunk of planned images (pcell / pfold set).
@@ -174,6 +160,30 @@ svdlut_status launch_prep(const LaunchArgs<N> &a, int sm_count, cudaStream_t s)
     return launch_pdl(prep_kernel<N>, dim3(kLutCtas * a.n + fold_ctas), dim3(kPrepThreads), smem, s, pa);
 }
 
+// Whether the precomputed tables are worth their launch for planned args on
+// `ctas` CTAs.  Without them a CTA folds its blocks' raw grids itself, K times
+// the loads of the folded slices; that takes longer from about 9000 loads a
+// CTA on, while the launch of prep_kernel and the wait for it cost about 4 us
+// whatever the size: 64 images of 256 x 256 with 17-vertex grids (5 K loads)
+// take 84 us without and 91 with, 16 of 480 x 640 with grids at 1/8 resolution
+// (12 K) 92 and 92, a 4K frame (18 K) 99 and 95.  Only the factors that
+// copy_factors takes are built quickly in the CTAs.
+template <int N>
+bool tables_pay(const LaunchArgs<N> &a, int ctas)
+{
+    constexpr double kMaxLoads = 9216;
+    double loads = 0;
+    for (int i = 0; i < a.n; ++i) {
+        const ImgDesc &e = a.img[i];
+        const int nvx = span_bound(kTileW, e.W, e.Dsx), nvy = span_bound(e.BH, e.H, e.Dsy);
+        const int xcol = fold_floats(nvx, nvy, e.Dsc) + 2 * kTileW + ((2 * a.bh_max + 3) & ~3);
+        if (!fast_factors_ok(e) || xcol + fast_factor_floats(e.D) > a.scratch_floats) return true;
+        const int blocks = (i + 1 < a.n ? a.img[i + 1].block_begin : a.total_blocks) - e.block_begin;
+        loads += static_cast<double>(blocks) * e.K * (nvx * nvy + (nvx + nvy) * e.Dsc);
+    }
+    return loads > kMaxLoads * std::min(ctas, a.total_blocks);
+}
+
 // Launches apply_kernel for args whose blocks are already planned.  dx_mode
 // runs the pixel part of the adjoint (float images only).
 template <int N>
@@ -184,10 +194,9 @@ svdlut_status launch_apply(LaunchArgs<N> &a, size_t smem, svdlut_dtype dt, cudaS
     DeviceInfo di;
     svdlut_status st = device_info(&di);
     if (st != SVDLUT_OK) return st;
-    if (dx_mode) return launch_apply_t<IoF32, N, true>(a, smem, di.sm_count, di.max_smem_optin, di.device, s, grid);
-    return dt == SVDLUT_F32
-               ? launch_apply_t<IoF32, N, false>(a, smem, di.sm_count, di.max_smem_optin, di.device, s, grid)
-               : launch_apply_t<IoU8, N, false>(a, smem, di.sm_count, di.max_smem_optin, di.device, s, grid);
+    if (dx_mode) return launch_io<IoF32, N, true>(a, smem, di, s, grid);
+    return dt == SVDLUT_F32 ? launch_io<IoF32, N, false>(a, smem, di, s, grid)
+                            : launch_io<IoU8, N, false>(a, smem, di, s, grid);
 }
 
 }  // namespace svdlut

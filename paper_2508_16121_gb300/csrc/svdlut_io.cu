@@ -100,9 +100,7 @@ svdlut_status run_io(const svdlut_dims *dims, const svdlut_params *params, int B
         if ((st = plan_uniform(a, di.sm_count, static_cast<size_t>(di.max_smem_optin), &smem)) != SVDLUT_OK)
             return st;
         if (a.total_blocks <= 0) continue;
-        if ((st = launch_apply_t<IO, kPlainChunk, false>(a, smem, di.sm_count, di.max_smem_optin, di.device, s, 0)) !=
-            SVDLUT_OK)
-            return st;
+        if ((st = launch_io<IO, kPlainChunk, false>(a, smem, di, s, 0)) != SVDLUT_OK) return st;
     }
     return SVDLUT_OK;
 }
