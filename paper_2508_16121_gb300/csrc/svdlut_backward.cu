@@ -115,6 +115,7 @@ __device__ __forceinline__ bool merge_equal_keys(int key, float (&v)[12])
 __global__ void __launch_bounds__(kLutThreads, 1)
     lut_grad_kernel(BwdArgs a, float *__restrict__ lut_part, float *__restrict__ sums_part)
 {
+    pdl_enter();
     extern __shared__ __align__(16) float sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = warp / 3, pair = warp - grp * 3;
@@ -387,6 +388,7 @@ __device__ __forceinline__ void spread_columns(const float *row, const float *co
 __global__ void __launch_bounds__(kGridThreads, 1)
     grid_grad_kernel(BwdArgs a, GridPlan gp, float *__restrict__ grid_part)
 {
+    pdl_enter();
     extern __shared__ __align__(16) float sm[];
     __shared__ int wy_off[kGridGroups], wy_n[kGridGroups];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = gp.groups * 3, nthr = nw * 32;
@@ -679,6 +681,7 @@ struct FinArgs {
 __global__ void __launch_bounds__(kFinThreads)
     lut_finalize_kernel(FinArgs f, const float *__restrict__ lut_part, const float *__restrict__ sums_part)
 {
+    pdl_enter();
     extern __shared__ __align__(16) float sm[];
     const int cp = blockIdx.x, b = blockIdx.y, c = cp / 3, pair = cp - c * 3;
     const int D = f.D, R = f.R, DD = D * D, DR = D * R;
@@ -796,6 +799,7 @@ __host__ __device__ inline int grid_plane_size(int plane, int Dsx, int Dsy, int 
 __global__ void __launch_bounds__(kGRThreads, 4)
     grid_reduce_kernel(GridRed g, const float *__restrict__ grid_part)
 {
+    pdl_enter();
     extern __shared__ int gtab[];  // ylo[bands], nvy[bands], xlo[strips], nvx[strips]
     __shared__ float red[kGRThreads / 32][kMaxKK];
     const GridPlan &gp = g.gp;
@@ -887,6 +891,7 @@ struct GridWsum {
 
 __global__ void grid_wsum_kernel(GridWsum f, const float *__restrict__ wpart, const float *__restrict__ sums_part)
 {
+    pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;  // (b, k, entry)
     if (t >= f.B * f.K * 4) return;
     const int q = t & 3, bk = t >> 2, b = bk / f.K, k = bk - b * f.K;
@@ -1070,6 +1075,36 @@ static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, in
     return SVDLUT_OK;
 }
 
+// The dx pass, N images per launch; with `tables` (B times prep_img bytes) the
+// per-image tables may be precomputed once (prep_kernel) instead of in every
+// CTA.  One launch for 64 images of 256 x 256 instead of four of 16: the
+// blocks of a launch fill the SMs once, and three tails and table launches go.
+template <int N>
+static svdlut_status dx_chunks(const svdlut_dims *dims, const svdlut_params *params, int B, int H, int W,
+                               const float *x, const float *dy, float *dx, char *tables, size_t prep_img,
+                               const DeviceInfo &di, cudaStream_t s)
+{
+    svdlut_status st = SVDLUT_OK;
+    for (int b0 = 0; b0 < B; b0 += N) {
+        LaunchArgs<N> a{};
+        a.n = std::min(N, B - b0);
+        for (int i = 0; i < a.n; ++i) {
+            a.img[i] = make_desc(dims, params, b0 + i, H, W, SVDLUT_F32, x, dx);
+            a.img[i].dy = dy + static_cast<size_t>(b0 + i) * 3 * H * W;
+            a.img[i].vec = a.img[i].vec && aligned(a.img[i].dy, 16);
+            if (tables) set_prep_tables(a.img[i], dims, tables + static_cast<size_t>(b0 + i) * prep_img);
+        }
+        size_t smem = 0;
+        if ((st = plan_uniform(a, di.sm_count, static_cast<size_t>(di.max_smem_optin), &smem)) != SVDLUT_OK) return st;
+        if (tables && tables_pay(a, di.sm_count)) {
+            if ((st = launch_prep(a, di.sm_count, s)) != SVDLUT_OK) return st;
+            a.pre = 1;
+        }
+        if ((st = launch_apply(a, smem, SVDLUT_F32, s, 0, true)) != SVDLUT_OK) return st;
+    }
+    return SVDLUT_OK;
+}
+
 static svdlut_status check_backward_args(const svdlut_dims *dims, const svdlut_params *params, int B, int H,
                                          int W, const float *x, const float *dy)
 {
@@ -1131,29 +1166,13 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
         return fail(SVDLUT_ERR_WORKSPACE, "workspace of %zu bytes needed (got %zu)", pl.total, ws ? ws_bytes : 0);
     if (have_ws && !aligned(ws, 256)) return fail(SVDLUT_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
 
-    // 1. dx through the forward kernel's adjoint mode; with a workspace, the
-    // per-image tables are precomputed once (prep_kernel) instead of in
-    // every CTA
+    // 1. dx through the forward kernel's adjoint mode, up to 16 images per
+    // launch, or 64 when the batch is larger
     if (dx) {
-        for (int b0 = 0; b0 < B; b0 += kPlainChunk) {
-            LaunchArgs<kPlainChunk> a{};
-            a.n = std::min(kPlainChunk, B - b0);
-            for (int i = 0; i < a.n; ++i) {
-                a.img[i] = make_desc(dims, params, b0 + i, H, W, SVDLUT_F32, x, dx);
-                a.img[i].dy = dy + static_cast<size_t>(b0 + i) * 3 * H * W;
-                a.img[i].vec = a.img[i].vec && aligned(a.img[i].dy, 16);
-                if (have_ws)
-                    set_prep_tables(a.img[i], dims,
-                                    static_cast<char *>(ws) + pl.off_prep + static_cast<size_t>(b0 + i) * pl.prep_img);
-            }
-            size_t smem = 0;
-            if ((st = plan_uniform(a, di.sm_count, smem_limit, &smem)) != SVDLUT_OK) return st;
-            if (have_ws) {
-                if ((st = launch_prep(a, di.sm_count, s)) != SVDLUT_OK) return st;
-                a.pre = 1;
-            }
-            if ((st = launch_apply(a, smem, SVDLUT_F32, s, 0, true)) != SVDLUT_OK) return st;
-        }
+        char *tables = have_ws ? static_cast<char *>(ws) + pl.off_prep : nullptr;
+        st = B > kPlainChunk ? dx_chunks<kRaggedMax>(dims, params, B, H, W, x, dy, dx, tables, pl.prep_img, di, s)
+                             : dx_chunks<kPlainChunk>(dims, params, B, H, W, x, dy, dx, tables, pl.prep_img, di, s);
+        if (st != SVDLUT_OK) return st;
     }
     if (!want_lut && !want_grid) return SVDLUT_OK;
     char *w = static_cast<char *>(ws);
@@ -1190,18 +1209,21 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
     if (pl.grid_smem + 256 > static_cast<size_t>(di.max_smem_optin) || pl.lut_smem > static_cast<size_t>(di.max_smem_optin))
         return fail(SVDLUT_ERR_UNSUPPORTED, "adjoint tables do not fit in shared memory");
     // 2. LUT pass (also produces the dy channel sums used by every bias)
-    lut_grad_kernel<<<dim3(pl.P, B), kLutThreads, pl.lut_smem, s>>>(a, lut_part, sums_part);
-    SVDLUT_CUDA_TRY(cudaGetLastError());
+    if ((st = launch_pdl(lut_grad_kernel, dim3(pl.P, B), dim3(kLutThreads), pl.lut_smem, s, a, lut_part, sums_part)) !=
+        SVDLUT_OK)
+        return st;
     if (want_lut) {
         FinArgs f{params->U, params->S, params->V, params->lut_w, g.dU, g.dS, g.dV, g.dlut_w,
                   dims->D_t, dims->rank, pl.P};
         const size_t fsm = sizeof(float) * (2 * dims->D_t * dims->D_t + dims->D_t * dims->rank + kFinThreads / 32);
-        lut_finalize_kernel<<<dim3(9, B), kFinThreads, fsm, s>>>(f, lut_part, sums_part);
-        SVDLUT_CUDA_TRY(cudaGetLastError());
+        if ((st = launch_pdl(lut_finalize_kernel, dim3(9, B), dim3(kFinThreads), fsm, s, f,
+                             static_cast<const float *>(lut_part), static_cast<const float *>(sums_part))) != SVDLUT_OK)
+            return st;
     }
     if (want_grid) {
-        grid_grad_kernel<<<dim3(pl.gp.nblk, B), pl.gp.groups * 3 * 32, pl.grid_smem, s>>>(a, pl.gp, grid_part);
-        SVDLUT_CUDA_TRY(cudaGetLastError());
+        if ((st = launch_pdl(grid_grad_kernel, dim3(pl.gp.nblk, B), dim3(pl.gp.groups * 3 * 32), pl.grid_smem, s, a,
+                             pl.gp, grid_part)) != SVDLUT_OK)
+            return st;
         GridRed r{};
         r.B = B;
         r.H = H;
@@ -1233,13 +1255,15 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
             if (rsm + sizeof(float) * (kGRThreads / 32) * kMaxKK > static_cast<size_t>(di.max_smem_optin))
                 return fail(SVDLUT_ERR_UNSUPPORTED, "too many column strips and row bands for the grid reduction");
         }
-        grid_reduce_kernel<<<dim3(3 * (pl.sl[0] + pl.sl[1] + pl.sl[2]), B), kGRThreads, rsm, s>>>(r, grid_part);
-        SVDLUT_CUDA_TRY(cudaGetLastError());
+        if ((st = launch_pdl(grid_reduce_kernel, dim3(3 * (pl.sl[0] + pl.sl[1] + pl.sl[2]), B), dim3(kGRThreads), rsm, s,
+                             r, static_cast<const float *>(grid_part))) != SVDLUT_OK)
+            return st;
         if (g.dgrid_w) {
             GridWsum f{B, dims->K, pl.P, pl.smax, {pl.sl[0], pl.sl[1], pl.sl[2]}, g.dgrid_w};
             const int n = B * dims->K * 4;
-            grid_wsum_kernel<<<(n + 255) / 256, 256, 0, s>>>(f, wpart, sums_part);
-            SVDLUT_CUDA_TRY(cudaGetLastError());
+            if ((st = launch_pdl(grid_wsum_kernel, dim3((n + 255) / 256), dim3(256), 0, s, f,
+                                 static_cast<const float *>(wpart), static_cast<const float *>(sums_part))) != SVDLUT_OK)
+                return st;
         }
     }
     return SVDLUT_OK;
