@@ -47,9 +47,11 @@ struct BwdArgs {
 // ---------------------------------------------------------------------------
 // LUT gradients: G^c_p[i][j] = sum_px dy_c * bilinear weight of vertex (i, j)
 // at (x_alpha, x_beta) for pair p = (alpha, beta).
-// grid (P, B); CTA (p, b) owns the rows [p H / P, (p+1) H / P) of image b.
-// Its work is the sequence of (64-column strip, row) pairs, strip by strip;
-// row group g takes the g-th share of it (equal to within one row).
+// The work is the sequence of (image, 64-column strip, row) triples; CTA g of G
+// takes the g-th share of it (equal to within one row), one image's part of it
+// after another, and row group g of the CTA the g-th share of a part.  Shares
+// of the whole batch, not of an image: 64 images of 256 x 256 on 152 SMs take
+// 152 CTAs, where whole CTAs per image left 24 SMs idle.
 // Warp (pair q, group g) walks down the rows of its share; lane l takes
 // columns l and l + 32 and keeps, per column, the twelve corner sums (four
 // corners, three channels) of its current cell in registers: while the cell
@@ -72,7 +74,8 @@ struct BwdArgs {
 // warps update in turns: 660, 440 and 563 us, the hand-over's latency; 12
 // warps of this kernel: 580, 323, 460 us; the queue for every batch: 671,
 // 282, 491 us.
-// Output: lut_part[b][p][c][pair][D*D], sums_part[b][p][c] (sum of dy_c).
+// Output per part of CTA g and image b, in slot g + b (lut_slots): lut_part
+// [slot][c][pair][D*D], sums_part[slot][c] (sum of dy_c).
 // ---------------------------------------------------------------------------
 constexpr int kLutGroups = 5, kLutWarps = 3 * kLutGroups;
 constexpr int kLutThreads = kLutWarps * 32;
@@ -86,6 +89,18 @@ __host__ __device__ inline int lut_table_floats(int D) { return (3 * D * D + 3) 
 __host__ __device__ inline size_t lut_grad_smem(int D)
 {
     return sizeof(float) * (kLutWarps * (static_cast<size_t>(lut_table_floats(D)) + kLutQueueFloats) + 4 * kLutGroups);
+}
+
+// Shares of the LUT pass: work units [share(g), share(g + 1)) belong to CTA g.
+__host__ __device__ inline long long lut_share(long long units, int G, int g) { return units * g / G; }
+// The slots of image b's parts, one per CTA that holds some of it: a CTA's next
+// image, and an image's next CTA, is the next slot.
+__host__ __device__ inline void lut_slots(long long per_image, int B, int G, int b, int &s0, int &s1)
+{
+    const long long U = per_image * B;
+    auto owner = [&](long long u) { return static_cast<int>(((u + 1) * G + U - 1) / U - 1); };
+    s0 = owner(per_image * b) + b;
+    s1 = owner(per_image * (b + 1) - 1) + b + 1;
 }
 
 // Adds the 12 sums of lanes with equal keys (key < 0: none) into the lowest
@@ -120,184 +135,190 @@ __global__ void __launch_bounds__(kLutThreads, 1)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = warp / 3, pair = warp - grp * 3;
     const int A = pair == 2 ? 1 : 0, Bx = pair == 0 ? 1 : 2;  // axes of the pair
-    const int P = gridDim.x, p = blockIdx.x, b = blockIdx.y;
     const int D = a.D, DD = D * D, tf = lut_table_floats(D);
     float *tab = sm + warp * tf;  // [D][D][3] of this warp's pair
     float4 *qv = reinterpret_cast<float4 *>(sm + kLutWarps * tf + warp * kLutQueueFloats);  // [3][kLutQueue]
     int *qk = reinterpret_cast<int *>(qv + 3 * kLutQueue);                                   // [kLutQueue]
     float *sums = sm + kLutWarps * (tf + kLutQueueFloats);                                   // [kLutGroups][4]
-    for (int e = threadIdx.x; e < kLutWarps * tf / 4; e += kLutThreads)
-        reinterpret_cast<float4 *>(sm)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-
-    const int r0 = static_cast<int>((static_cast<long long>(a.H) * p) / P);
-    const int r1 = static_cast<int>((static_cast<long long>(a.H) * (p + 1)) / P);
     const size_t plane = static_cast<size_t>(a.H) * a.W;
-    const float *xa = a.x + (static_cast<size_t>(b) * 3 + A) * plane, *xbp = a.x + (static_cast<size_t>(b) * 3 + Bx) * plane;
-    const float *gb = a.dy + static_cast<size_t>(b) * 3 * plane;
     const float fD1 = static_cast<float>(D - 1), fD2 = static_cast<float>(D - 2);
-    const int nrows = r1 - r0, strips = (a.W + kLutTileW - 1) / kLutTileW;
-    const long long T = static_cast<long long>(strips) * nrows;
-    const long long t0 = T * grp / kLutGroups, t1 = T * (grp + 1) / kLutGroups;
-    const int my_rows = static_cast<int>(t1 - t0);
+    const int strips = (a.W + kLutTileW - 1) / kLutTileW;
+    const long long per_image = static_cast<long long>(strips) * a.H;
+    const long long c1 = lut_share(per_image * a.B, gridDim.x, blockIdx.x + 1);
+    for (long long c0 = lut_share(per_image * a.B, gridDim.x, blockIdx.x); c0 < c1;) {
+        // this image's part of the share: units [u0, u1) of image b
+        const int b = static_cast<int>(c0 / per_image);
+        const long long u0 = c0 - b * per_image, u1 = min(c1 - b * per_image, per_image);
+        c0 = b * per_image + u1;
+        for (int e = threadIdx.x; e < kLutWarps * tf / 4; e += kLutThreads)
+            reinterpret_cast<float4 *>(sm)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncthreads();
 
-    float acc[2][12];  // [column][corner * 3 + channel]
-    int acc_key[2] = {-1, -1};
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int i = 0; i < 12; ++i) acc[k][i] = 0.f;
-    int qn = 0;  // queued sums
-    float dysum[3] = {0.f, 0.f, 0.f};
+        const float *xa = a.x + (static_cast<size_t>(b) * 3 + A) * plane, *xbp = a.x + (static_cast<size_t>(b) * 3 + Bx) * plane;
+        const float *gb = a.dy + static_cast<size_t>(b) * 3 * plane;
+        const long long t0 = u0 + (u1 - u0) * grp / kLutGroups, t1 = u0 + (u1 - u0) * (grp + 1) / kLutGroups;
+        const int my_rows = static_cast<int>(t1 - t0);
 
-    // adds the sums of the lanes with key >= 0 to the table
-    auto add_batch = [&](int key, float (&v)[12]) {
-        const bool leader = merge_equal_keys(key, v);
-        const int off[4] = {0, 3 * D, 3, 3 * D + 3};
+        float acc[2][12];  // [column][corner * 3 + channel]
+        int acc_key[2] = {-1, -1};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (leader) {
-                float *t = tab + key * 3 + off[q];
-                const float u0 = t[0], u1 = t[1], u2 = t[2];
-                t[0] = u0 + v[q * 3];
-                t[1] = u1 + v[q * 3 + 1];
-                t[2] = u2 + v[q * 3 + 2];
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int i = 0; i < 12; ++i) acc[k][i] = 0.f;
+        int qn = 0;  // queued sums
+        float dysum[3] = {0.f, 0.f, 0.f};
+
+        // adds the sums of the lanes with key >= 0 to the table
+        auto add_batch = [&](int key, float (&v)[12]) {
+            const bool leader = merge_equal_keys(key, v);
+            const int off[4] = {0, 3 * D, 3, 3 * D + 3};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (leader) {
+                    float *t = tab + key * 3 + off[q];
+                    const float u0 = t[0], u1 = t[1], u2 = t[2];
+                    t[0] = u0 + v[q * 3];
+                    t[1] = u1 + v[q * 3 + 1];
+                    t[2] = u2 + v[q * 3 + 2];
+                }
+                __syncwarp();
             }
+        };
+        auto drain = [&]() {
+            float w[12];
+            int k = -1;
             __syncwarp();
-        }
-    };
-    auto drain = [&]() {
-        float w[12];
-        int k = -1;
-        __syncwarp();
-        if (lane < qn) {
-            const float4 q0 = qv[lane], q1 = qv[kLutQueue + lane], q2 = qv[2 * kLutQueue + lane];
-            w[0] = q0.x;
-            w[1] = q0.y;
-            w[2] = q0.z;
-            w[3] = q0.w;
-            w[4] = q1.x;
-            w[5] = q1.y;
-            w[6] = q1.z;
-            w[7] = q1.w;
-            w[8] = q2.x;
-            w[9] = q2.y;
-            w[10] = q2.z;
-            w[11] = q2.w;
-            k = qk[lane];
-        } else {
+            if (lane < qn) {
+                const float4 q0 = qv[lane], q1 = qv[kLutQueue + lane], q2 = qv[2 * kLutQueue + lane];
+                w[0] = q0.x;
+                w[1] = q0.y;
+                w[2] = q0.z;
+                w[3] = q0.w;
+                w[4] = q1.x;
+                w[5] = q1.y;
+                w[6] = q1.z;
+                w[7] = q1.w;
+                w[8] = q2.x;
+                w[9] = q2.y;
+                w[10] = q2.z;
+                w[11] = q2.w;
+                k = qk[lane];
+            } else {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) w[i] = 0.f;
-        }
-        qn = 0;
-        add_batch(k, w);
-    };
-    // the sums v of the lanes with key >= 0 are finished
-    auto finish = [&](int key, float (&v)[12]) {
-        const unsigned int done = __ballot_sync(0xffffffffu, key >= 0);
-        const int cnt = __popc(done);
-        if (cnt >= kLutDirect) {
-            add_batch(key, v);
-            return;
-        }
-        if (qn + cnt > kLutQueue) drain();
-        if (key >= 0) {
-            const int s = qn + __popc(done & ((1u << lane) - 1u));
-            qv[s] = make_float4(v[0], v[1], v[2], v[3]);
-            qv[kLutQueue + s] = make_float4(v[4], v[5], v[6], v[7]);
-            qv[2 * kLutQueue + s] = make_float4(v[8], v[9], v[10], v[11]);
-            qk[s] = key;
-        }
-        qn += cnt;
-    };
+                for (int i = 0; i < 12; ++i) w[i] = 0.f;
+            }
+            qn = 0;
+            add_batch(k, w);
+        };
+        // the sums v of the lanes with key >= 0 are finished
+        auto finish = [&](int key, float (&v)[12]) {
+            const unsigned int done = __ballot_sync(0xffffffffu, key >= 0);
+            const int cnt = __popc(done);
+            if (cnt >= kLutDirect) {
+                add_batch(key, v);
+                return;
+            }
+            if (qn + cnt > kLutQueue) drain();
+            if (key >= 0) {
+                const int s = qn + __popc(done & ((1u << lane) - 1u));
+                qv[s] = make_float4(v[0], v[1], v[2], v[3]);
+                qv[kLutQueue + s] = make_float4(v[4], v[5], v[6], v[7]);
+                qv[2 * kLutQueue + s] = make_float4(v[8], v[9], v[10], v[11]);
+                qk[s] = key;
+            }
+            qn += cnt;
+        };
 
-    struct Row {
-        float pa[2], pb[2], g[3][2];
-        int n;  // this lane's columns: 0, 1 or 2
-    };
-    // rows are loaded one ahead of their use, from the cursor (strip, row)
-    int ls = static_cast<int>(t0 / nrows), lr = static_cast<int>(t0 - ls * static_cast<long long>(nrows)), loaded = 0;
-    auto load = [&](Row &o) {
-        const int x = ls * kLutTileW + lane;
-        o.n = loaded < my_rows ? (x < a.W) + (x + 32 < a.W) : 0;
-        const size_t off = static_cast<size_t>(r0 + lr) * a.W + x;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const bool in = k < o.n;
-            o.pa[k] = in ? __ldcs(xa + off + 32 * k) : 0.f;
-            o.pb[k] = in ? __ldcs(xbp + off + 32 * k) : 0.f;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) o.g[c][k] = in ? __ldcs(gb + c * plane + off + 32 * k) : 0.f;
-        }
-        ++loaded;
-        if (++lr == nrows) {
-            lr = 0;
-            ++ls;
-        }
-    };
-    Row cur, nxt;
-    load(cur);
-    for (int r = 0; r < my_rows; ++r) {
-        load(nxt);
-        float da[2], db[2];
-        int key[2];
-        bool change[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int ia = cell_of(__saturatef(cur.pa[k]), fD1, fD2, da[k]);
-            const int ib = cell_of(__saturatef(cur.pb[k]), fD1, fD2, db[k]);
-            key[k] = ia * D + ib;
-            change[k] = k < cur.n && key[k] != acc_key[k];
-        }
-        if (__any_sync(0xffffffffu, change[0] || change[1])) {
+        struct Row {
+            float pa[2], pb[2], g[3][2];
+            int n;  // this lane's columns: 0, 1 or 2
+        };
+        // rows are loaded one ahead of their use, from the cursor (strip, row)
+        int ls = static_cast<int>(t0 / a.H), lr = static_cast<int>(t0 - ls * static_cast<long long>(a.H)), loaded = 0;
+        auto load = [&](Row &o) {
+            const int x = ls * kLutTileW + lane;
+            o.n = loaded < my_rows ? (x < a.W) + (x + 32 < a.W) : 0;
+            const size_t off = static_cast<size_t>(lr) * a.W + x;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                finish(change[k] ? acc_key[k] : -1, acc[k]);
-                if (change[k]) {
+                const bool in = k < o.n;
+                o.pa[k] = in ? __ldcs(xa + off + 32 * k) : 0.f;
+                o.pb[k] = in ? __ldcs(xbp + off + 32 * k) : 0.f;
 #pragma unroll
-                    for (int i = 0; i < 12; ++i) acc[k][i] = 0.f;
-                    acc_key[k] = key[k];
+                for (int c = 0; c < 3; ++c) o.g[c][k] = in ? __ldcs(gb + c * plane + off + 32 * k) : 0.f;
+            }
+            ++loaded;
+            if (++lr == a.H) {
+                lr = 0;
+                ++ls;
+            }
+        };
+        Row cur, nxt;
+        load(cur);
+        for (int r = 0; r < my_rows; ++r) {
+            load(nxt);
+            float da[2], db[2];
+            int key[2];
+            bool change[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int ia = cell_of(__saturatef(cur.pa[k]), fD1, fD2, da[k]);
+                const int ib = cell_of(__saturatef(cur.pb[k]), fD1, fD2, db[k]);
+                key[k] = ia * D + ib;
+                change[k] = k < cur.n && key[k] != acc_key[k];
+            }
+            if (__any_sync(0xffffffffu, change[0] || change[1])) {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    finish(change[k] ? acc_key[k] : -1, acc[k]);
+                    if (change[k]) {
+#pragma unroll
+                        for (int i = 0; i < 12; ++i) acc[k][i] = 0.f;
+                        acc_key[k] = key[k];
+                    }
                 }
             }
-        }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float w[4] = {(1.f - da[k]) * (1.f - db[k]), da[k] * (1.f - db[k]), (1.f - da[k]) * db[k], da[k] * db[k]};
+            for (int k = 0; k < 2; ++k) {
+                const float w[4] = {(1.f - da[k]) * (1.f - db[k]), da[k] * (1.f - db[k]), (1.f - da[k]) * db[k], da[k] * db[k]};
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                dysum[c] += cur.g[c][k];
-                // a column outside the image adds nothing (its dy is 0)
+                for (int c = 0; c < 3; ++c) {
+                    dysum[c] += cur.g[c][k];
+                    // a column outside the image adds nothing (its dy is 0)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[k][q * 3 + c] = fmaf(cur.g[c][k], w[q], acc[k][q * 3 + c]);
+                    for (int q = 0; q < 4; ++q) acc[k][q * 3 + c] = fmaf(cur.g[c][k], w[q], acc[k][q * 3 + c]);
+                }
             }
+            cur = nxt;
         }
-        cur = nxt;
-    }
-    finish(acc_key[0], acc[0]);
-    finish(acc_key[1], acc[1]);
-    drain();
+        finish(acc_key[0], acc[0]);
+        finish(acc_key[1], acc[1]);
+        drain();
 
-    // sum of dy_c: the pair-0 warps' totals (every pair warp of a group sees the same pixels)
+        // sum of dy_c: the pair-0 warps' totals (every pair warp of a group sees the same pixels)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) dysum[c] = warp_sum(dysum[c]);
-    if (lane == 0 && pair == 0) {
+        for (int c = 0; c < 3; ++c) dysum[c] = warp_sum(dysum[c]);
+        if (lane == 0 && pair == 0) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) sums[grp * 4 + c] = dysum[c];
-    }
-    __syncthreads();
-    // CTA partial [c][pair][vertex]: sum the groups in order
-    float *out = lut_part + (static_cast<size_t>(b) * P + p) * 9 * DD;
-    for (int e = threadIdx.x; e < 9 * DD; e += kLutThreads) {
-        const int c = e / (3 * DD), r = e - c * 3 * DD, q = r / DD, vtx = r - q * DD;
-        float s = 0.f;
+            for (int c = 0; c < 3; ++c) sums[grp * 4 + c] = dysum[c];
+        }
+        __syncthreads();
+        // CTA partial [c][pair][vertex]: sum the groups in order
+        const size_t slot = static_cast<size_t>(blockIdx.x) + b;
+        float *out = lut_part + slot * 9 * DD;
+        for (int e = threadIdx.x; e < 9 * DD; e += kLutThreads) {
+            const int c = e / (3 * DD), r = e - c * 3 * DD, q = r / DD, vtx = r - q * DD;
+            float s = 0.f;
 #pragma unroll
-        for (int g = 0; g < kLutGroups; ++g) s += sm[(g * 3 + q) * tf + vtx * 3 + c];
-        out[e] = s;
-    }
-    if (threadIdx.x < 3) {
-        float s = 0.f;
-        for (int g = 0; g < kLutGroups; ++g) s += sums[g * 4 + threadIdx.x];
-        sums_part[(static_cast<size_t>(b) * P + p) * 3 + threadIdx.x] = s;
+            for (int g = 0; g < kLutGroups; ++g) s += sm[(g * 3 + q) * tf + vtx * 3 + c];
+            out[e] = s;
+        }
+        if (threadIdx.x < 3) {
+            float s = 0.f;
+            for (int g = 0; g < kLutGroups; ++g) s += sums[g * 4 + threadIdx.x];
+            sums_part[slot * 3 + threadIdx.x] = s;
+        }
+        __syncthreads();  // the tables are cleared for the next image
     }
 }
 
@@ -675,7 +696,8 @@ __device__ inline float block_sum(float v, float *red)
 struct FinArgs {
     const float *U, *S, *V, *lw;
     float *dU, *dS, *dV, *dlw;
-    int D, R, P;
+    int D, R, B, G;       // G: CTAs of the LUT pass
+    long long per_image;  // its work units per image
 };
 
 __global__ void __launch_bounds__(kFinThreads)
@@ -685,6 +707,8 @@ __global__ void __launch_bounds__(kFinThreads)
     extern __shared__ __align__(16) float sm[];
     const int cp = blockIdx.x, b = blockIdx.y, c = cp / 3, pair = cp - c * 3;
     const int D = f.D, R = f.R, DD = D * D, DR = D * R;
+    int s0, s1;  // the image's slots
+    lut_slots(f.per_image, f.B, f.G, b, s0, s1);
     float *G = sm, *T = sm + DD, *Q = T + DD, *red = Q + DR;  // Q[i][r] = sum_j dT[i][j] V[j][r]
     const float *U = f.U + (static_cast<size_t>(b) * 9 + cp) * DR;
     const float *V = f.V + (static_cast<size_t>(b) * 9 + cp) * DR;
@@ -692,7 +716,7 @@ __global__ void __launch_bounds__(kFinThreads)
     const float w = f.lw[static_cast<size_t>(b) * 12 + c * 4 + pair];
     for (int e = threadIdx.x; e < DD; e += kFinThreads) {
         float s = 0.f;
-        for (int p = 0; p < f.P; ++p) s += lut_part[((static_cast<size_t>(b) * f.P + p) * 9 + cp) * DD + e];
+        for (int q = s0; q < s1; ++q) s += lut_part[(static_cast<size_t>(q) * 9 + cp) * DD + e];
         G[e] = s;
         const int i = e / D, j = e - i * D;
         float tv = 0.f;
@@ -708,7 +732,7 @@ __global__ void __launch_bounds__(kFinThreads)
         f.dlw[static_cast<size_t>(b) * 12 + c * 4 + pair] = dw;
         if (pair == 0) {
             float s = 0.f;
-            for (int p = 0; p < f.P; ++p) s += sums_part[(static_cast<size_t>(b) * f.P + p) * 3 + c];
+            for (int q = s0; q < s1; ++q) s += sums_part[static_cast<size_t>(q) * 3 + c];
             f.dlw[static_cast<size_t>(b) * 12 + c * 4 + 3] = s;
         }
     }
@@ -884,9 +908,10 @@ __global__ void __launch_bounds__(kGRThreads, 4)
 // dgrid_w[b][k] = (the slice partials of each plane summed in order, the sum
 // of dy_{k mod 3} over the image from the LUT pass partials: the bias).
 struct GridWsum {
-    int B, K, P, smax;
+    int B, K, G, smax;
     int sl[3];
     float *dgw;
+    long long per_image;
 };
 
 __global__ void grid_wsum_kernel(GridWsum f, const float *__restrict__ wpart, const float *__restrict__ sums_part)
@@ -900,7 +925,9 @@ __global__ void grid_wsum_kernel(GridWsum f, const float *__restrict__ wpart, co
         const float *p = wpart + ((static_cast<size_t>(b) * 3 + q) * f.K + k) * f.smax;
         for (int i = 0; i < f.sl[q]; ++i) s += p[i];
     } else {
-        for (int p = 0; p < f.P; ++p) s += sums_part[(static_cast<size_t>(b) * f.P + p) * 3 + k % 3];
+        int s0, s1;
+        lut_slots(f.per_image, f.B, f.G, b, s0, s1);
+        for (int i = s0; i < s1; ++i) s += sums_part[static_cast<size_t>(i) * 3 + k % 3];
     }
     f.dgw[static_cast<size_t>(bk) * 4 + q] = s;
 }
@@ -909,7 +936,8 @@ __global__ void grid_wsum_kernel(GridWsum f, const float *__restrict__ wpart, co
 // host planning and workspace
 // ---------------------------------------------------------------------------
 struct BwdPlan {
-    int P;             // LUT-pass CTAs per image
+    int G;             // LUT-pass CTAs
+    long long units;   // its work units per image
     size_t lut_smem;   // bytes
     GridPlan gp;
     size_t grid_smem;  // bytes
@@ -950,15 +978,16 @@ static bool grid_density_ok(int BH, int nvx, int H, int Dsy, int Dsc, size_t sme
     return sizeof(float) * kWarps * warp + 256 <= smem_limit;
 }
 
-// Workspace layout of a plan whose P and gp are set.
+// Workspace layout of a plan whose G and gp are set.
 static void layout_backward(const svdlut_dims *d, int B, BwdPlan *pl)
 {
     const int D = d->D_t;
     size_t off = 0;
     pl->off_lut = off;
-    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->P * 9 * D * D);
+    const size_t slots = static_cast<size_t>(B) + pl->G - 1;
+    off = align256(off + sizeof(float) * slots * 9 * D * D);
     pl->off_sums = off;
-    off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->P * 3);
+    off = align256(off + sizeof(float) * slots * 3);
     pl->off_grid = off;
     off = align256(off + sizeof(float) * static_cast<size_t>(B) * pl->gp.nblk * pl->gp.blk_stride);
     pl->smax = 1;
@@ -974,28 +1003,26 @@ static void layout_backward(const svdlut_dims *d, int B, BwdPlan *pl)
     pl->total = off;
 }
 
-// LUT pass: CTAs per image, at most max_p (one CTA per SM); estimated time =
-// waves x (rows a group walks: its share of strips x rows, + a fixed cost of
-// about 16 rows per CTA: clearing the tables, writing the partial) + a row's
-// time per 24 partials that lut_finalize_kernel sums.
-static int plan_lut_ctas(int B, int H, int W, int sm_count, int max_p)
+// LUT pass: CTAs, at most max_g (one per SM); estimated time = rows a group
+// walks (its share of the batch's strips x rows, + a fixed cost of about 16 rows
+// per CTA: clearing the tables, writing the partial) + a row's time per 24
+// partials of an image that lut_finalize_kernel sums.
+static int plan_lut_ctas(int B, long long units, int max_g)
 {
-    const long long strips = (W + kLutTileW - 1) / kLutTileW;
+    const long long U = units * B;
     long long best_cost = -1;
     int best = 1;
-    for (int P = 1; P <= std::min({H, 4 * sm_count, max_p}); ++P) {
-        const long long waves = (static_cast<long long>(B) * P + sm_count - 1) / sm_count;
-        const long long rows = (H + P - 1) / P;
-        const long long cost = 24 * waves * ((strips * rows + kLutGroups - 1) / kLutGroups + 16) + P;
+    for (int G = 1; G <= std::min<long long>(U, max_g); ++G) {
+        const long long cost = 24 * (((U + G - 1) / G + kLutGroups - 1) / kLutGroups + 16) + (G + B - 1) / B;
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
-            best = P;
+            best = G;
         }
     }
     return best;
 }
 
-// Grid pass of a plan whose P is set: blocks of 128 x BH with as many row
+// Grid pass of a plan whose G is set: blocks of 128 x BH with as many row
 // groups as fit; bands minimise waves x (rows a warp walks + a fixed cost of
 // about 8 rows per block: clearing the tables, summing the warps, writing the
 // partial), ties go to the better-filled waves, and plans within
@@ -1050,24 +1077,25 @@ static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, in
 {
     pl->lut_smem = lut_grad_smem(d->D_t);
     if (pl->lut_smem > smem_limit) return fail(SVDLUT_ERR_UNSUPPORTED, "D_t=%d too large for the adjoint", d->D_t);
-    pl->P = plan_lut_ctas(B, H, W, sm_count, H);
+    pl->units = static_cast<long long>((W + kLutTileW - 1) / kLutTileW) * H;
+    pl->G = plan_lut_ctas(B, pl->units, sm_count);
     if (!plan_grid(d, B, H, W, sm_count, smem_limit, false, pl))
         return fail(SVDLUT_ERR_UNSUPPORTED, "grid vertices too dense for the adjoint's blocks");
     if (pl->total > kNoAllocScratchBytes) {
         // stay within svdlut_backward_noalloc's scratch where fewer LUT CTAs
         // and the smallest grid plan do
         BwdPlan q = *pl;
-        q.P = 1;
+        q.G = 1;
         plan_grid(d, B, H, W, sm_count, smem_limit, true, &q);
         if (q.total <= kNoAllocScratchBytes) {
-            const size_t per = sizeof(float) * static_cast<size_t>(B) * (9 * d->D_t * d->D_t + 3);
-            q.P = std::min(pl->P, static_cast<int>(1 + (kNoAllocScratchBytes - q.total) / per));
+            const size_t per = sizeof(float) * (9 * static_cast<size_t>(d->D_t) * d->D_t + 3);
+            q.G = static_cast<int>(std::min<size_t>(pl->G, 1 + (kNoAllocScratchBytes - q.total) / per));
             layout_backward(d, B, &q);
             while (q.total > kNoAllocScratchBytes) {  // the parts' alignment
-                --q.P;
+                --q.G;
                 layout_backward(d, B, &q);
             }
-            q.P = plan_lut_ctas(B, H, W, sm_count, q.P);
+            q.G = plan_lut_ctas(B, q.units, q.G);
             plan_grid(d, B, H, W, sm_count, smem_limit, false, &q);
             *pl = q;
         }
@@ -1209,12 +1237,12 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
     if (pl.grid_smem + 256 > static_cast<size_t>(di.max_smem_optin) || pl.lut_smem > static_cast<size_t>(di.max_smem_optin))
         return fail(SVDLUT_ERR_UNSUPPORTED, "adjoint tables do not fit in shared memory");
     // 2. LUT pass (also produces the dy channel sums used by every bias)
-    if ((st = launch_pdl(lut_grad_kernel, dim3(pl.P, B), dim3(kLutThreads), pl.lut_smem, s, a, lut_part, sums_part)) !=
+    if ((st = launch_pdl(lut_grad_kernel, dim3(pl.G), dim3(kLutThreads), pl.lut_smem, s, a, lut_part, sums_part)) !=
         SVDLUT_OK)
         return st;
     if (want_lut) {
         FinArgs f{params->U, params->S, params->V, params->lut_w, g.dU, g.dS, g.dV, g.dlut_w,
-                  dims->D_t, dims->rank, pl.P};
+                  dims->D_t, dims->rank, B, pl.G, pl.units};
         const size_t fsm = sizeof(float) * (2 * dims->D_t * dims->D_t + dims->D_t * dims->rank + kFinThreads / 32);
         if ((st = launch_pdl(lut_finalize_kernel, dim3(9, B), dim3(kFinThreads), fsm, s, f,
                              static_cast<const float *>(lut_part), static_cast<const float *>(sums_part))) != SVDLUT_OK)
@@ -1259,7 +1287,7 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
                              r, static_cast<const float *>(grid_part))) != SVDLUT_OK)
             return st;
         if (g.dgrid_w) {
-            GridWsum f{B, dims->K, pl.P, pl.smax, {pl.sl[0], pl.sl[1], pl.sl[2]}, g.dgrid_w};
+            GridWsum f{B, dims->K, pl.G, pl.smax, {pl.sl[0], pl.sl[1], pl.sl[2]}, g.dgrid_w, pl.units};
             const int n = B * dims->K * 4;
             if ((st = launch_pdl(grid_wsum_kernel, dim3((n + 255) / 256), dim3(256), 0, s, f,
                                  static_cast<const float *>(wpart), static_cast<const float *>(sums_part))) != SVDLUT_OK)

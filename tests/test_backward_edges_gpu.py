@@ -75,3 +75,12 @@ def test_lut_gradients_are_bitwise_repeatable():
         again = sv.backward(xt, pt, dy)
         for k in first:
             assert torch.equal(first[k], again[k]), k
+
+
+# shares of the LUT pass that end inside images, hold several whole ones, are
+# one row, or are fewer than the SMs (batch, H, W)
+@pytest.mark.parametrize("B,H,W", [(7, 45, 70), (160, 3, 65), (3, 1, 1), (64, 40, 64), (5, 171, 129)])
+def test_lut_shares_across_images(B, H, W):
+    d = si.Dims(17, 4, 3, 3, 3, 5)
+    x, p = si.make_batch(900 + B, B, H, W, d)
+    check(x, p, si.make_upstream(901 + B, x.shape), d)
