@@ -24,36 +24,76 @@ from ._lib import SvdlutError  # noqa: F401
 PARAM_NAMES = ("U", "S", "V", "lut_w", "g_xy", "g_xc", "g_yc", "grid_w")
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+def _sizes_of(params):
+    U, gxy = params["U"].shape, params["g_xy"].shape
+    return U[-2], U[-1], gxy[-3], gxy[-1], gxy[-2], params["g_xc"].shape[-1]
 
 
 def dims_of(params) -> _lib.Dims:
     """Infer (D_t, rank, K, Dsx, Dsy, Dsc) from parameter tensor shapes
     (per-image [3,3,D,R] or batched [B,3,3,D,R] U)."""
-    U, gxy, gxc = params["U"], params["g_xy"], params["g_xc"]
-    D, R = U.shape[-2], U.shape[-1]
-    K, Dsy, Dsx = gxy.shape[-3], gxy.shape[-2], gxy.shape[-1]
-    Dsc = gxc.shape[-1]
-    return _lib.Dims(D, R, K, Dsx, Dsy, Dsc)
+    return _lib.Dims(*_sizes_of(params))
+
+
+class _Sizes:
+    """What follows from the transform's sizes alone: the ABI's dims (only
+    read), the shape and count of each parameter of one image, and the bytes of
+    its precomputed tables."""
+
+    def __init__(self, sizes):
+        D, R, K, Dsx, Dsy, Dsc = sizes
+        self.dims = _lib.Dims(*sizes)
+        shapes = ((3, 3, D, R), (3, 3, R), (3, 3, D, R), (3, 4), (K, Dsy, Dsx), (K, Dsx, Dsc), (K, Dsy, Dsc), (K, 4))
+        self.params = tuple((n, w, _numel(w)) for n, w in zip(PARAM_NAMES, shapes))
+        self.table_bytes = None
+
+
+_sizes = {}  # sizes -> _Sizes; a few hundred at most
+
+
+def _sizes_entry(sizes):
+    e = _sizes.get(sizes)
+    if e is None:
+        if len(_sizes) >= 256:
+            _sizes.clear()
+        e = _sizes[sizes] = _Sizes(sizes)
+    return e
+
+
+def _pointers(params, B, entry):
+    f32 = _torch().float32
+    ptrs = []
+    for n, want, count in entry.params:
+        t = params[n]
+        if t.dtype != f32 or not t.is_cuda or not t.is_contiguous():
+            raise ValueError(f"param {n} must be a contiguous float32 CUDA tensor")
+        shape = t.shape
+        if shape[-len(want):] != want or t.numel() != B * count:
+            raise ValueError(f"param {n}: shape {tuple(shape)} does not match {want} x B={B}")
+        ptrs.append(t.data_ptr() if count else None)
+    return _lib.Params(*ptrs)
 
 
 def _param_struct(params, B, d):
-    torch = _torch()
-    shapes = {"U": (3, 3, d.D_t, d.rank), "S": (3, 3, d.rank), "V": (3, 3, d.D_t, d.rank),
-              "lut_w": (3, 4), "g_xy": (d.K, d.Dsy, d.Dsx), "g_xc": (d.K, d.Dsx, d.Dsc),
-              "g_yc": (d.K, d.Dsy, d.Dsc), "grid_w": (d.K, 4)}
-    ptrs = {}
-    for n in PARAM_NAMES:
-        t = params[n]
-        if t.dtype != torch.float32 or not t.is_cuda or not t.is_contiguous():
-            raise ValueError(f"param {n} must be a contiguous float32 CUDA tensor")
-        want = shapes[n]
-        if tuple(t.shape[-len(want):]) != want or t.numel() != B * _numel(want):
-            raise ValueError(f"param {n}: shape {tuple(t.shape)} does not match {want} x B={B}")
-        ptrs[n] = t.data_ptr() if t.numel() else None
-    return _lib.Params(**ptrs)
+    return _pointers(params, B, _sizes_entry((d.D_t, d.rank, d.K, d.Dsx, d.Dsy, d.Dsc)))
+
+
+def _dims_params(params, B):
+    """The ABI's dims and parameter pointers of a parameter dict for B images,
+    and the sizes' entry."""
+    e = _sizes_entry(_sizes_of(params))
+    return e.dims, _pointers(params, B, e), e
 
 
 def _numel(s):
@@ -64,9 +104,10 @@ def _numel(s):
 
 
 def _stream_ptr(stream=None):
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def apply(x, params, out=None, stream=None, ctas=None, workspace=True):
@@ -93,34 +134,31 @@ def apply(x, params, out=None, stream=None, ctas=None, workspace=True):
     else:
         raise ValueError("x must be float32 or uint8")
     B, _, H, W = xb.shape
-    d = dims_of(params)
-    p = _param_struct(params, B, d)
+    d, p, sizes = _dims_params(params, B)
     y = torch.empty_like(xb) if out is None else (out.unsqueeze(0) if squeeze else out)
-    if y.shape != xb.shape or y.dtype != xb.dtype or not y.is_contiguous():
+    if out is not None and (y.shape != xb.shape or y.dtype != xb.dtype or not y.is_contiguous()):
         raise ValueError("out must match x in shape and dtype")
     lib = _lib.load()
     if workspace is not False:
-        need = lib.svdlut_apply_workspace_size(ctypes.byref(d), B)
+        if sizes.table_bytes is None:
+            sizes.table_bytes = lib.svdlut_apply_workspace_size(d, 1)
+        need = B * sizes.table_bytes
         if workspace is True:
             ws = _stream_workspace(torch, need, xb.device, stream)
+            ws_bytes = need
         else:
             ws = workspace
-            if not ws.is_cuda or ws.dtype != torch.uint8 or ws.numel() < need:
+            ws_bytes = ws.numel()
+            if not ws.is_cuda or ws.dtype != torch.uint8 or ws_bytes < need:
                 raise ValueError(f"workspace must be a uint8 CUDA tensor of at least {need} bytes")
-        cfg = _lib.LaunchCfg(0, int(ctas or 0), 0)
-        _lib.check(lib.svdlut_apply_ws(ctypes.byref(d), ctypes.byref(p), B, H, W, dt,
-                                       ctypes.c_void_p(xb.data_ptr()), ctypes.c_void_p(y.data_ptr()),
-                                       ctypes.byref(cfg), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+        cfg = _lib.LaunchCfg(0, int(ctas), 0) if ctas else None
+        _lib.check(lib.svdlut_apply_ws(d, p, B, H, W, dt, xb.data_ptr(), y.data_ptr(), cfg, ws.data_ptr(), ws_bytes,
                                        _stream_ptr(stream)))
     elif ctas is None:
-        _lib.check(lib.svdlut_apply(ctypes.byref(d), ctypes.byref(p), B, H, W, dt,
-                                    ctypes.c_void_p(xb.data_ptr()), ctypes.c_void_p(y.data_ptr()),
-                                    _stream_ptr(stream)))
+        _lib.check(lib.svdlut_apply(d, p, B, H, W, dt, xb.data_ptr(), y.data_ptr(), _stream_ptr(stream)))
     else:
-        cfg = _lib.LaunchCfg(0, int(ctas), 0)
-        _lib.check(lib.svdlut_apply_cfg(ctypes.byref(d), ctypes.byref(p), B, H, W, dt,
-                                        ctypes.c_void_p(xb.data_ptr()), ctypes.c_void_p(y.data_ptr()),
-                                        ctypes.byref(cfg), _stream_ptr(stream)))
+        _lib.check(lib.svdlut_apply_cfg(d, p, B, H, W, dt, xb.data_ptr(), y.data_ptr(), _lib.LaunchCfg(0, int(ctas), 0),
+                                        _stream_ptr(stream)))
     return y[0] if squeeze else y
 
 
@@ -175,11 +213,9 @@ def apply_io(x, params, in_format, out_format, out=None, stream=None):
         yb, _, Ho, Wo = _pix_tensor(out, out_format, "out")
         if (yb.shape[0], Ho, Wo) != (B, H, W):
             raise ValueError("out must hold the same images as x")
-    d = dims_of(params)
-    p = _param_struct(params, B, d)
-    _lib.check(_lib.load().svdlut_apply_io(ctypes.byref(d), ctypes.byref(p), B, H, W, PIXEL_FORMATS[in_format][0],
-                                           ctypes.c_void_p(xb.data_ptr()), PIXEL_FORMATS[out_format][0],
-                                           ctypes.c_void_p(yb.data_ptr()), _stream_ptr(stream)))
+    d, p, _ = _dims_params(params, B)
+    _lib.check(_lib.load().svdlut_apply_io(d, p, B, H, W, PIXEL_FORMATS[in_format][0], xb.data_ptr(),
+                                           PIXEL_FORMATS[out_format][0], yb.data_ptr(), _stream_ptr(stream)))
     return yb[0] if single else yb
 
 
@@ -208,8 +244,7 @@ def apply_host(x, params, out=None, stream=None):
     else:
         raise ValueError("x must be float32 or uint8")
     B, _, H, W = xb.shape
-    d = dims_of(params)
-    p = _param_struct(params, B, d)
+    d, p, _ = _dims_params(params, B)
     y = torch.empty(xb.shape, dtype=xb.dtype, pin_memory=True) if out is None else (out.unsqueeze(0) if squeeze else out)
     if y.shape != xb.shape or y.dtype != xb.dtype or y.is_cuda or not y.is_contiguous():
         raise ValueError("out must be a host tensor matching x in shape and dtype")
@@ -219,20 +254,19 @@ def apply_host(x, params, out=None, stream=None):
     if not (xb.is_pinned() and y.is_pinned()):  # pinned frames are used in place, no workspace
         need = lib.svdlut_apply_host_workspace_size(B, H, W, dt)
         dev = next(iter(params.values())).device
-        key = (str(dev), sp.value)  # one workspace per device and stream: calls on one stream are ordered
+        key = (str(dev), sp)  # one workspace per device and stream: calls on one stream are ordered
         ws = _host_ws.get(key)
         if ws is None or ws.numel() < need:
             ws = torch.empty(need, dtype=torch.uint8, device=dev)
             _host_ws[key] = ws
         ws_ptr, ws_bytes = ws.data_ptr(), ws.numel()
-    _lib.check(lib.svdlut_apply_host(ctypes.byref(d), ctypes.byref(p), B, H, W, dt, ctypes.c_void_p(xb.data_ptr()),
-                                     ctypes.c_void_p(y.data_ptr()), ctypes.c_void_p(ws_ptr), ws_bytes, sp))
+    _lib.check(lib.svdlut_apply_host(d, p, B, H, W, dt, xb.data_ptr(), y.data_ptr(), ws_ptr, ws_bytes, sp))
     return y[0] if squeeze else y
 
 
 def original_workspace_bytes(params, B, H, W):
     """Device workspace of apply_original for B images of H x W."""
-    return int(_lib.load().svdlut_apply_original_workspace_size(ctypes.byref(dims_of(params)), B, H, W))
+    return int(_lib.load().svdlut_apply_original_workspace_size(dims_of(params), B, H, W))
 
 
 def apply_original(x, params, fusion, out=None, workspace=None, stream=None):
@@ -246,8 +280,7 @@ def apply_original(x, params, fusion, out=None, workspace=None, stream=None):
     if xb.dim() != 4 or xb.shape[1] != 3 or xb.dtype != torch.float32 or not xb.is_cuda or not xb.is_contiguous():
         raise ValueError("x must be a contiguous float32 CUDA tensor [B,3,H,W] or [3,H,W]")
     B, _, H, W = xb.shape
-    d = dims_of(params)
-    p = _param_struct(params, B, d)
+    d, p, _ = _dims_params(params, B)
     nf = 3 * (d.K + 3) + 3
     f = fusion.reshape(-1, nf)
     if f.shape[0] == 1 and B > 1:
@@ -257,12 +290,11 @@ def apply_original(x, params, fusion, out=None, workspace=None, stream=None):
         raise ValueError(f"fusion must hold {nf} floats per image on the GPU")
     y = torch.empty_like(xb) if out is None else (out.unsqueeze(0) if squeeze else out)
     lib = _lib.load()
-    need = lib.svdlut_apply_original_workspace_size(ctypes.byref(d), B, H, W)
+    need = lib.svdlut_apply_original_workspace_size(d, B, H, W)
     ws = workspace if workspace is not None and workspace.numel() >= need else \
         torch.empty(need, dtype=torch.uint8, device=xb.device)
-    _lib.check(lib.svdlut_apply_original(ctypes.byref(d), ctypes.byref(p), ctypes.c_void_p(f.data_ptr()), B, H, W,
-                                         ctypes.c_void_p(xb.data_ptr()), ctypes.c_void_p(y.data_ptr()),
-                                         ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream_ptr(stream)))
+    _lib.check(lib.svdlut_apply_original(d, p, f.data_ptr(), B, H, W, xb.data_ptr(), y.data_ptr(),
+                                         ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return y[0] if squeeze else y
 
 
@@ -296,9 +328,8 @@ def lut3d_apply(x, lut3d, out=None, workspace=None, stream=None):
     need = lib.svdlut_lut3d_workspace_size(D, B)
     ws = workspace if workspace is not None and workspace.numel() >= need else \
         torch.empty(need, dtype=torch.uint8, device=xb.device)
-    _lib.check(lib.svdlut_lut3d_apply(D, ctypes.c_void_p(t.data_ptr()), B, H, W, ctypes.c_void_p(xb.data_ptr()),
-                                      ctypes.c_void_p(y.data_ptr()), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
-                                      _stream_ptr(stream)))
+    _lib.check(lib.svdlut_lut3d_apply(D, t.data_ptr(), B, H, W, xb.data_ptr(), y.data_ptr(), ws.data_ptr(),
+                                      ws.numel(), _stream_ptr(stream)))
     return y[0] if squeeze else y
 
 
@@ -311,8 +342,8 @@ def lut3d_fit2d(lut3d, stream=None):
     B, D = t.shape[0], t.shape[-1]
     tables = torch.empty(B, 3, 3, D, D, dtype=torch.float32, device=t.device)
     rms = torch.empty(B, 3, dtype=torch.float32, device=t.device)
-    _lib.check(_lib.load().svdlut_lut3d_fit2d(D, ctypes.c_void_p(t.data_ptr()), B, ctypes.c_void_p(tables.data_ptr()),
-                                              ctypes.c_void_p(rms.data_ptr()), _stream_ptr(stream)))
+    _lib.check(_lib.load().svdlut_lut3d_fit2d(D, t.data_ptr(), B, tables.data_ptr(), rms.data_ptr(),
+                                              _stream_ptr(stream)))
     return tables, rms
 
 
@@ -363,26 +394,23 @@ def backward(x, params, dy, want=("dx",) + tuple("d" + n for n in PARAM_NAMES), 
     if gb.shape != xb.shape or not xb.is_contiguous() or not gb.is_contiguous():
         raise ValueError("dy must be contiguous and shaped like x")
     B, _, H, W = xb.shape
-    d = dims_of(params)
-    p = _param_struct(params, B, d)
+    d, p, _ = _dims_params(params, B)
     out = {}
     ptrs = {}
     for n in PARAM_NAMES:
-        if "d" + n in want:
-            t = torch.empty_like(params[n])
-            out["d" + n] = t
-            ptrs["d" + n] = t.data_ptr() if t.numel() else None
+        dn = "d" + n
+        if dn in want:
+            t = out[dn] = torch.empty_like(params[n])
+            ptrs[dn] = t.data_ptr() if t.numel() else None
     g = _lib.Grads(**ptrs)
     dx = torch.empty_like(xb) if "dx" in want else None
     lib = _lib.load()
-    need = lib.svdlut_backward_workspace_size(ctypes.byref(d), B, H, W)
+    need = lib.svdlut_backward_workspace_size(d, B, H, W)
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(max(need, 1), dtype=torch.uint8, device=xb.device)
-    _lib.check(lib.svdlut_backward(ctypes.byref(d), ctypes.byref(p), B, H, W, ctypes.c_void_p(xb.data_ptr()),
-                                   ctypes.c_void_p(gb.data_ptr()),
-                                   ctypes.c_void_p(dx.data_ptr()) if dx is not None else None,
-                                   ctypes.byref(g), ctypes.c_void_p(workspace.data_ptr()), workspace.numel(),
-                                   _stream_ptr(stream)))
+    _lib.check(lib.svdlut_backward(d, p, B, H, W, xb.data_ptr(), gb.data_ptr(),
+                                   dx.data_ptr() if dx is not None else None, g, workspace.data_ptr(),
+                                   workspace.numel(), _stream_ptr(stream)))
     if dx is not None:
         out["dx"] = dx[0] if squeeze else dx
     return out
@@ -452,7 +480,7 @@ class Batch:
                 raise ValueError("all images (and outputs) must share one dtype and match in shape")
             d = dims_of(p)
             self.imgs[i] = _lib.Image(x.shape[1], x.shape[2], d, _param_struct(p, 1, d),
-                                      ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(y.data_ptr()))
+                                      x.data_ptr(), y.data_ptr())
         lib = _lib.load()
         need = lib.svdlut_batched_tables_workspace_size(self.imgs, n) if tables else \
             lib.svdlut_batched_workspace_size(n)
@@ -461,9 +489,8 @@ class Batch:
 
     def run(self, stream=None):
         lib = _lib.load()
-        cfg = ctypes.byref(self.cfg) if self.cfg is not None else None
-        _lib.check(lib.svdlut_apply_batched(self.imgs, len(self.xs), self.dtype, cfg,
-                                            ctypes.c_void_p(self.ws.data_ptr()), self.ws.numel(),
+        _lib.check(lib.svdlut_apply_batched(self.imgs, len(self.xs), self.dtype, self.cfg,
+                                            self.ws.data_ptr(), self.ws.numel(),
                                             _stream_ptr(stream)))
         return self.outs
 
@@ -500,7 +527,7 @@ class Batch:
         best = _lib.LaunchCfg()
         ms = ctypes.c_float()
         _lib.check(lib.svdlut_autotune_batched(self.imgs, len(self.xs), self.dtype,
-                                               ctypes.c_void_p(self.ws.data_ptr()), self.ws.numel(),
+                                               self.ws.data_ptr(), self.ws.numel(),
                                                _stream_ptr(stream), reps, ctypes.byref(best), ctypes.byref(ms)))
         self.cfg = best
         if path:
@@ -563,10 +590,10 @@ class Generator:
             raise ValueError("x must be a contiguous float32 [B,3,H,W] with B <= max_batch")
         out = out if out is not None else self.empty_params(B)
         lib = _lib.load()
-        _lib.check(lib.svdlut_generator_forward(self.K, ctypes.c_void_p(self.weights.data_ptr()), B, H, W,
-                                                ctypes.c_void_p(x.data_ptr()), ctypes.byref(self._ptrs(out)),
+        _lib.check(lib.svdlut_generator_forward(self.K, self.weights.data_ptr(), B, H, W,
+                                                x.data_ptr(), self._ptrs(out),
                                                 int(bool(training)), ctypes.c_uint64(seed),
-                                                ctypes.c_void_p(self.ws.data_ptr()), self.ws.numel(),
+                                                self.ws.data_ptr(), self.ws.numel(),
                                                 _stream_ptr(stream)))
         self.last = (B, int(bool(training)), int(seed))
         return out
@@ -578,10 +605,10 @@ class Generator:
         B, training, seed = self.last
         dw = dweights if dweights is not None else torch.empty_like(self.weights)
         lib = _lib.load()
-        _lib.check(lib.svdlut_generator_backward(self.K, ctypes.c_void_p(self.weights.data_ptr()), B,
-                                                 ctypes.byref(self._ptrs(dparams)), ctypes.c_void_p(dw.data_ptr()),
+        _lib.check(lib.svdlut_generator_backward(self.K, self.weights.data_ptr(), B,
+                                                 self._ptrs(dparams), dw.data_ptr(),
                                                  training, ctypes.c_uint64(seed),
-                                                 ctypes.c_void_p(self.ws.data_ptr()), self.ws.numel(),
+                                                 self.ws.data_ptr(), self.ws.numel(),
                                                  _stream_ptr(stream)))
         return dw
 
@@ -589,8 +616,8 @@ class Generator:
 def adam_step(weights, grads, m, v, step, lr=1e-4, beta1=0.9, beta2=0.999, eps=1e-8, stream=None):
     """One Adam step on FP32 CUDA tensors (svdlut_generator_adam)."""
     lib = _lib.load()
-    _lib.check(lib.svdlut_generator_adam(ctypes.c_void_p(weights.data_ptr()), ctypes.c_void_p(grads.data_ptr()),
-                                         ctypes.c_void_p(m.data_ptr()), ctypes.c_void_p(v.data_ptr()), weights.numel(),
+    _lib.check(lib.svdlut_generator_adam(weights.data_ptr(), grads.data_ptr(),
+                                         m.data_ptr(), v.data_ptr(), weights.numel(),
                                          lr, beta1, beta2, eps, int(step), _stream_ptr(stream)))
 
 
@@ -613,10 +640,10 @@ def cie94(y, target, weight=1.0, dy=None, accumulate=False, ws=None, stream=None
     B, _, H, W = yb.shape
     loss = torch.empty((), dtype=torch.float32, device=y.device)
     ws = ws if ws is not None else torch.empty(4096, dtype=torch.uint8, device=y.device)
-    _lib.check(_lib.load().svdlut_cie94(ctypes.c_void_p(yb.data_ptr()), ctypes.c_void_p(tb.data_ptr()), B, H, W,
-                                        float(weight), ctypes.c_void_p(dy.data_ptr()) if dy is not None else None,
-                                        int(bool(accumulate)), ctypes.c_void_p(loss.data_ptr()),
-                                        ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream_ptr(stream)))
+    _lib.check(_lib.load().svdlut_cie94(yb.data_ptr(), tb.data_ptr(), B, H, W,
+                                        float(weight), dy.data_ptr() if dy is not None else None,
+                                        int(bool(accumulate)), loss.data_ptr(),
+                                        ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return loss
 
 
@@ -626,8 +653,8 @@ def mse(y, target, dy=None, ws=None, stream=None):
     loss = torch.empty((), dtype=torch.float32, device=y.device)
     ws = ws if ws is not None else torch.empty(4096, dtype=torch.uint8, device=y.device)
     lib = _lib.load()
-    _lib.check(lib.svdlut_mse(ctypes.c_void_p(y.data_ptr()), ctypes.c_void_p(target.data_ptr()), y.numel(),
-                              ctypes.c_void_p(dy.data_ptr()) if dy is not None else None,
-                              ctypes.c_void_p(loss.data_ptr()), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+    _lib.check(lib.svdlut_mse(y.data_ptr(), target.data_ptr(), y.numel(),
+                              dy.data_ptr() if dy is not None else None,
+                              loss.data_ptr(), ws.data_ptr(), ws.numel(),
                               _stream_ptr(stream)))
     return loss

@@ -56,6 +56,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = False):
     """Load libsvdlut.so.  Raises if it is missing (no fallback path)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
