@@ -677,9 +677,12 @@ __global__ void __launch_bounds__(kGridThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// LUT finalize: one CTA per (table c*3+pair, image).
+// LUT finalize: one CTA per (table c*3+pair, image).  The image's partials are
+// summed in up to kFinParts contiguous parts, side by side, kFinBatch loads at a
+// time, then the parts in order: two images' 152 partials on 18 CTAs were bound
+// by the latency of one chain of loads per vertex (76 us at 2 x 342x628).
 // ---------------------------------------------------------------------------
-constexpr int kFinThreads = 256;
+constexpr int kFinMaxThreads = 1024, kFinParts = 8, kFinBatch = 8;
 
 __device__ inline float block_sum(float v, float *red)
 {
@@ -689,7 +692,7 @@ __device__ inline float block_sum(float v, float *red)
     if (lane == 0) red[warp] = v;
     __syncthreads();
     float s = 0.f;
-    for (int w = 0; w < kFinThreads / 32; ++w) s += red[w];
+    for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) s += red[w];
     return s;
 }
 
@@ -700,85 +703,109 @@ struct FinArgs {
     long long per_image;  // its work units per image
 };
 
-__global__ void __launch_bounds__(kFinThreads)
+__host__ __device__ inline int fin_smem_floats(int D, int R) { return kFinParts * D * D + 3 * D * R + R + kFinMaxThreads / 32; }
+
+__global__ void __launch_bounds__(kFinMaxThreads)
     lut_finalize_kernel(FinArgs f, const float *__restrict__ lut_part, const float *__restrict__ sums_part)
 {
     pdl_enter();
     extern __shared__ __align__(16) float sm[];
+    const int nthr = blockDim.x;
     const int cp = blockIdx.x, b = blockIdx.y, c = cp / 3, pair = cp - c * 3;
     const int D = f.D, R = f.R, DD = D * D, DR = D * R;
     int s0, s1;  // the image's slots
     lut_slots(f.per_image, f.B, f.G, b, s0, s1);
-    float *G = sm, *T = sm + DD, *Q = T + DD, *red = Q + DR;  // Q[i][r] = sum_j dT[i][j] V[j][r]
-    const float *U = f.U + (static_cast<size_t>(b) * 9 + cp) * DR;
-    const float *V = f.V + (static_cast<size_t>(b) * 9 + cp) * DR;
-    const float *S = f.S + (static_cast<size_t>(b) * 9 + cp) * R;
+    float *G = sm;  // [kFinParts][DD]: the parts' sums, then G = the gradient of the table in part 0
+    float *U = sm + kFinParts * DD, *V = U + DR, *Q = V + DR, *S = Q + DR, *red = S + R;  // Q[i][r] = sum_j dT[i][j] V[j][r]
+    const size_t t = static_cast<size_t>(b) * 9 + cp;
+    for (int e = threadIdx.x; e < DR; e += nthr) {
+        U[e] = f.U[t * DR + e];
+        V[e] = f.V[t * DR + e];
+    }
+    if (threadIdx.x < R) S[threadIdx.x] = f.S[t * R + threadIdx.x];
     const float w = f.lw[static_cast<size_t>(b) * 12 + c * 4 + pair];
-    for (int e = threadIdx.x; e < DD; e += kFinThreads) {
+    const int n = s1 - s0, parts = max(1, min(kFinParts, n / kFinBatch));
+    for (int it = threadIdx.x; it < parts * DD; it += nthr) {
+        const int part = it / DD, e = it - part * DD;
+        const int q1 = s0 + n * (part + 1) / parts;
+        const float *src = lut_part + cp * DD + e;
         float s = 0.f;
-        for (int q = s0; q < s1; ++q) s += lut_part[(static_cast<size_t>(q) * 9 + cp) * DD + e];
-        G[e] = s;
+        for (int q = s0 + n * part / parts; q < q1; q += kFinBatch) {
+            float v[kFinBatch];
+#pragma unroll
+            for (int u = 0; u < kFinBatch; ++u) v[u] = q + u < q1 ? src[static_cast<size_t>(q + u) * 9 * DD] : 0.f;
+#pragma unroll
+            for (int u = 0; u < kFinBatch; ++u) s += v[u];
+        }
+        G[it] = s;
+    }
+    __syncthreads();
+    // G, and dw = <G, T>
+    float part = 0.f;
+    for (int e = threadIdx.x; e < DD; e += nthr) {
+        float g = G[e];
+        for (int p = 1; p < parts; ++p) g += G[p * DD + e];
+        G[e] = g;
         const int i = e / D, j = e - i * D;
         float tv = 0.f;
         for (int r = 0; r < R; ++r) tv = fmaf(U[i * R + r] * S[r], V[j * R + r], tv);
-        T[e] = tv;
+        part = fmaf(g, tv, part);
     }
-    __syncthreads();
-    // dw = <G, T>
-    float part = 0.f;
-    for (int e = threadIdx.x; e < DD; e += kFinThreads) part = fmaf(G[e], T[e], part);
     const float dw = block_sum(part, red);
     if (threadIdx.x == 0 && f.dlw) {
         f.dlw[static_cast<size_t>(b) * 12 + c * 4 + pair] = dw;
         if (pair == 0) {
             float s = 0.f;
+#pragma unroll 8
             for (int q = s0; q < s1; ++q) s += sums_part[static_cast<size_t>(q) * 3 + c];
             f.dlw[static_cast<size_t>(b) * 12 + c * 4 + 3] = s;
         }
     }
-    // Q = (w G) V ; dU = Q diag(S) ; dS_r = sum_i U[i][r] Q[i][r]
-    for (int e = threadIdx.x; e < DR; e += kFinThreads) {
-        const int i = e / R, r = e - i * R;
+    // Q = (w G) V; dU = Q diag(S); dV = (w G)^T U diag(S): items 0 .. DR - 1 and DR .. 2 DR - 1
+    for (int it = threadIdx.x; it < 2 * DR; it += nthr) {
+        const bool vside = it >= DR;
+        const int e = vside ? it - DR : it, i = e / R, r = e - i * R;
+        const float *g = G + (vside ? i : i * D), *m = (vside ? U : V) + r;
+        const int gs = vside ? D : 1;
         float s = 0.f;
-        for (int j = 0; j < D; ++j) s = fmaf(G[i * D + j], V[j * R + r], s);
-        Q[e] = w * s;
-        if (f.dU) f.dU[(static_cast<size_t>(b) * 9 + cp) * DR + e] = w * s * S[r];
+#pragma unroll 8
+        for (int j = 0; j < D; ++j) s = fmaf(g[j * gs], m[j * R], s);
+        if (!vside) Q[e] = w * s;
+        float *out = vside ? f.dV : f.dU;
+        if (out) out[t * DR + e] = w * s * S[r];
     }
-    // dV = (w G)^T U diag(S)
-    if (f.dV)
-        for (int e = threadIdx.x; e < DR; e += kFinThreads) {
-            const int j = e / R, r = e - j * R;
-            float s = 0.f;
-            for (int i = 0; i < D; ++i) s = fmaf(G[i * D + j], U[i * R + r], s);
-            f.dV[(static_cast<size_t>(b) * 9 + cp) * DR + e] = w * s * S[r];
-        }
     __syncthreads();
+    // dS_r = sum_i U[i][r] Q[i][r]
     if (f.dS && threadIdx.x < R) {
         const int r = threadIdx.x;
         float s = 0.f;
         for (int i = 0; i < D; ++i) s = fmaf(U[i * R + r], Q[i * R + r], s);
-        f.dS[(static_cast<size_t>(b) * 9 + cp) * R + r] = s;
+        f.dS[t * R + r] = s;
     }
 }
 
 // ---------------------------------------------------------------------------
 // grid reduce and finalize, fused.  A CTA takes a slice of kGRChunk vertices
-// of one folded plane (xy, xc or yc) of one output channel c of one image.
-// Per vertex it sums the partials of the blocks whose footprint holds the
-// vertex (bands, then strips, in order), which is dF_c at that vertex; then
-// for every grid k with k mod 3 = c it writes dg^k_plane = w^k_plane dF_c
-// (Supp. Eqs. 21-22: grid k feeds channel k mod 3 with weight w^k_plane) and
-// adds dF_c g^k_plane to the CTA's partial of dgrid_w[k][plane].
-// grid_wsum_kernel sums those partials over the slices in order.
+// of the folded planes xy, xc or yc of one image, a thread one vertex of all
+// three output channels (their blocks and offsets are the same).  It sums the
+// partials of the blocks whose footprint holds the vertex (bands, then strips,
+// in order), which is dF_c at that vertex; then for every grid k, c = k mod 3,
+// it writes dg^k_plane = w^k_plane dF_c (Supp. Eqs. 21-22: grid k feeds channel
+// k mod 3 with weight w^k_plane), and the sum of dF_c g^k_plane over the slice
+// is a partial of dgrid_w[k][plane].  grid_wsum_kernel sums those over the
+// slices in order.  Bound by latency and by finding the blocks (divisions):
+// the partials of kGRBatch blocks are loaded, then added; one channel per
+// thread and one load after another took 41 us at 2 x 342x628 (22 bands) and
+// 47 at 8 x 1920x1080.
 // ---------------------------------------------------------------------------
-constexpr int kGRThreads = 256, kGRChunk = kGRThreads * 2;
-constexpr int kMaxKK = (kMaxK + 2) / 3;  // grids per output channel
+constexpr int kGRThreads = 512, kGRChunk = kGRThreads;
+constexpr int kGRBatch = 4;  // blocks in flight per vertex
 
 struct GridRed {
     int B, H, W, K, Dsx, Dsy, Dsc, strips;
     float rW1, rH1;
     GridPlan gp;
-    int sl[3];  // slices per channel plane: xy, xc, yc
+    int sl[3];  // slices per plane: xy, xc, yc
     int smax;   // max(sl)
     const float *gxy, *gxc, *gyc, *gw;
     float *dgxy, *dgxc, *dgyc;  // any may be null
@@ -820,20 +847,15 @@ __host__ __device__ inline int grid_plane_size(int plane, int Dsx, int Dsy, int 
     return plane == 0 ? Dsy * Dsx : (plane == 1 ? Dsx * Dsc : Dsy * Dsc);
 }
 
-__global__ void __launch_bounds__(kGRThreads, 4)
+__global__ void __launch_bounds__(kGRThreads, 3)
     grid_reduce_kernel(GridRed g, const float *__restrict__ grid_part)
 {
     pdl_enter();
-    extern __shared__ int gtab[];  // ylo[bands], nvy[bands], xlo[strips], nvx[strips]
-    __shared__ float red[kGRThreads / 32][kMaxKK];
+    extern __shared__ int gtab[];  // ylo[bands], nvy[bands], xlo[strips], nvx[strips]; then the warps' sums [][K]
     const GridPlan &gp = g.gp;
     const int b = blockIdx.y;
-    int q = blockIdx.x, plane = 0;  // blockIdx.x -> (plane, channel c, slice)
-    while (plane < 2 && q >= 3 * g.sl[plane]) {
-        q -= 3 * g.sl[plane];
-        ++plane;
-    }
-    const int c = q / g.sl[plane], slice = q - c * g.sl[plane];
+    int slice = blockIdx.x, plane = 0;  // blockIdx.x -> (plane, slice)
+    while (plane < 2 && slice >= g.sl[plane]) slice -= g.sl[plane++];
     int *ylo = gtab, *nvy = gtab + gp.bands, *xlo = nvy + gp.bands, *nvx = xlo + g.strips;
     for (int t = threadIdx.x; t < gp.bands + g.strips; t += kGRThreads) {
         if (t < gp.bands) {
@@ -850,58 +872,80 @@ __global__ void __launch_bounds__(kGRThreads, 4)
     const int n = grid_plane_size(plane, Dsx, Dsy, Dsc), ncol = plane == 0 ? Dsx : Dsc;
     const float *gsrc = plane == 0 ? g.gxy : (plane == 1 ? g.gxc : g.gyc);
     float *gdst = plane == 0 ? g.dgxy : (plane == 1 ? g.dgxc : g.dgyc);
-    const int oxc = 3 * gp.nvy * gp.nvx, oyc = oxc + 3 * gp.nvx * Dsc;  // plane offsets in a block partial
-    float acc[kMaxKK];
-#pragma unroll
-    for (int kk = 0; kk < kMaxKK; ++kk) acc[kk] = 0.f;
-    const int e1 = min(n, (slice + 1) * kGRChunk);
-    for (int e = slice * kGRChunk + threadIdx.x; e < e1; e += kGRThreads) {
+    const int e = slice * kGRChunk + threadIdx.x;
+    const bool in = e < n;
+    float s[3] = {0.f, 0.f, 0.f};
+    if (in) {
         // xy: (iy, ix); xc: (ix, j); yc: (iy, j)
         const int r = e / ncol, col = e - r * ncol;
-        const int iy = plane == 1 ? -1 : r, ix = plane == 0 ? col : (plane == 1 ? r : -1), j = col;
+        const int iy = plane == 1 ? -1 : r, ix = plane == 0 ? col : (plane == 1 ? r : -1);
         int s0 = 0, s1 = g.strips - 1, b0 = 0, b1 = gp.bands - 1;
         if (ix >= 0) cover_range(ix, g.W, Dsx, kTileW, g.strips, s0, s1);
         if (iy >= 0) cover_range(iy, g.H, Dsy, gp.BH, gp.bands, b0, b1);
-        float s = 0.f;
-        for (int bd = b0; bd <= b1; ++bd) {
-            const int yl = ylo[bd], ny = nvy[bd];
-            if (ny <= 0 || (iy >= 0 && (iy < yl || iy >= yl + ny))) continue;
-            for (int st = s0; st <= s1; ++st) {
-                const int xl = xlo[st];
-                if (ix >= 0 && (ix < xl || ix >= xl + nvx[st])) continue;
-                const float *bp = grid_part + (static_cast<size_t>(b) * gp.nblk + bd * g.strips + st) * gp.blk_stride;
-                if (plane == 0)
-                    s += bp[((iy - yl) * gp.nvx + (ix - xl)) * 3 + c];
-                else if (plane == 1)
-                    s += bp[oxc + (c * gp.nvx + (ix - xl)) * Dsc + j];
-                else
-                    s += bp[oyc + (c * gp.nvy + (iy - yl)) * Dsc + j];
+        // offset in a block partial of the block's first vertex, strides of the
+        // vertex and of the channel
+        const int oxc = 3 * gp.nvy * gp.nvx, oyc = oxc + 3 * gp.nvx * Dsc;
+        const int base = plane == 0 ? 0 : (plane == 1 ? oxc + col : oyc + col);
+        const int vy = plane == 0 ? 3 * gp.nvx : (plane == 1 ? 0 : Dsc), vx = plane == 0 ? 3 : (plane == 1 ? Dsc : 0);
+        const int vc = plane == 0 ? 1 : (plane == 1 ? gp.nvx * Dsc : gp.nvy * Dsc);
+        const int nb = (b1 - b0 + 1) * (s1 - s0 + 1);
+        const float *img = grid_part + static_cast<size_t>(b) * gp.nblk * gp.blk_stride + base;
+        int bd = b0, st = s0;
+        for (int t = 0; t < nb; t += kGRBatch) {
+            float v[kGRBatch][3];
+#pragma unroll
+            for (int u = 0; u < kGRBatch; ++u) {
+                v[u][0] = v[u][1] = v[u][2] = 0.f;
+                if (t + u < nb) {
+                    const int dy = iy - ylo[bd], dx = ix - xlo[st], ny = nvy[bd];
+                    if (ny > 0 && (iy < 0 || (dy >= 0 && dy < ny)) && (ix < 0 || (dx >= 0 && dx < nvx[st]))) {
+                        const float *bp = img + static_cast<size_t>(bd * g.strips + st) * gp.blk_stride + dy * vy + dx * vx;
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) v[u][c] = bp[c * vc];
+                    }
+                    if (++st > s1) {
+                        st = s0;
+                        ++bd;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kGRBatch; ++u)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) s[c] += v[u][c];
+        }
+    }
+    // the grids, three at a time (channels 0, 1, 2)
+    float *red = reinterpret_cast<float *>(gtab);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k0 = 0; k0 < K; k0 += 3) {
+        float gv[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int k = k0 + c;
+            gv[c] = 0.f;
+            if (k < K && in) {
+                const size_t bk = static_cast<size_t>(b) * K + k;
+                if (gdst) gdst[bk * n + e] = __ldg(g.gw + bk * 4 + plane) * s[c];
+                if (g.wpart) gv[c] = __ldg(gsrc + bk * n + e) * s[c];
             }
         }
+        if (!g.wpart) continue;
 #pragma unroll
-        for (int kk = 0; kk < kMaxKK; ++kk) {
-            const int k = c + 3 * kk;
-            if (k >= K) break;
-            const size_t o = (static_cast<size_t>(b) * K + k) * n + e;
-            if (gdst) gdst[o] = __ldg(g.gw + (static_cast<size_t>(b) * K + k) * 4 + plane) * s;
-            acc[kk] = fmaf(s, __ldg(gsrc + o), acc[kk]);
+        for (int c = 0; c < 3; ++c) {
+            const float t = warp_sum(gv[c]);
+            if (lane == 0 && k0 + c < K) red[warp * K + k0 + c] = t;
         }
     }
     if (!g.wpart) return;
-    // the CTA's partials of dgrid_w: warp butterflies, then the warps in order
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int kk = 0; kk < kMaxKK; ++kk) {
-        if (c + 3 * kk >= K) break;
-        const float v = warp_sum(acc[kk]);
-        if (lane == 0) red[warp][kk] = v;
-    }
     __syncthreads();
-    const int k = c + 3 * static_cast<int>(threadIdx.x);
-    if (static_cast<int>(threadIdx.x) < kMaxKK && k < K) {
-        float s = 0.f;
-        for (int w = 0; w < kGRThreads / 32; ++w) s += red[w][threadIdx.x];
-        g.wpart[((static_cast<size_t>(b) * 3 + plane) * K + k) * g.smax + slice] = s;
+    // the slice's partials of dgrid_w: the warps in order
+    if (static_cast<int>(threadIdx.x) < K) {
+        const int k = threadIdx.x;
+        float t = 0.f;
+        for (int w = 0; w < kGRThreads / 32; ++w) t += red[w * K + k];
+        g.wpart[((static_cast<size_t>(b) * 3 + plane) * K + k) * g.smax + slice] = t;
     }
 }
 
@@ -923,10 +967,12 @@ __global__ void grid_wsum_kernel(GridWsum f, const float *__restrict__ wpart, co
     float s = 0.f;
     if (q < 3) {
         const float *p = wpart + ((static_cast<size_t>(b) * 3 + q) * f.K + k) * f.smax;
+#pragma unroll 8
         for (int i = 0; i < f.sl[q]; ++i) s += p[i];
     } else {
         int s0, s1;
         lut_slots(f.per_image, f.B, f.G, b, s0, s1);
+#pragma unroll 8
         for (int i = s0; i < s1; ++i) s += sums_part[static_cast<size_t>(i) * 3 + k % 3];
     }
     f.dgw[static_cast<size_t>(bk) * 4 + q] = s;
@@ -1104,8 +1150,10 @@ static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, in
 }
 
 // The dx pass, N images per launch; with `tables` (B times prep_img bytes) the
-// per-image tables may be precomputed once (prep_kernel) instead of in every
-// CTA.  One launch for 64 images of 256 x 256 instead of four of 16: the
+// per-image tables are precomputed once (prep_kernel) instead of in every CTA:
+// the instance that builds them spills registers, and loses 1 to 5 % at most
+// sizes (77 -> 74 us for svdlut_backward at 2 x 224x106, 490 -> 477 at 11 x
+// 514x1392; 337 -> 341 at 64 x 256x256).  One launch for 64 images of 256 x 256 instead of four of 16: the
 // blocks of a launch fill the SMs once, and three tails and table launches go.
 template <int N>
 static svdlut_status dx_chunks(const svdlut_dims *dims, const svdlut_params *params, int B, int H, int W,
@@ -1124,7 +1172,7 @@ static svdlut_status dx_chunks(const svdlut_dims *dims, const svdlut_params *par
         }
         size_t smem = 0;
         if ((st = plan_uniform(a, di.sm_count, static_cast<size_t>(di.max_smem_optin), &smem)) != SVDLUT_OK) return st;
-        if (tables && tables_pay(a, di.sm_count)) {
+        if (tables) {
             if ((st = launch_prep(a, di.sm_count, s)) != SVDLUT_OK) return st;
             a.pre = 1;
         }
@@ -1243,8 +1291,8 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
     if (want_lut) {
         FinArgs f{params->U, params->S, params->V, params->lut_w, g.dU, g.dS, g.dV, g.dlut_w,
                   dims->D_t, dims->rank, B, pl.G, pl.units};
-        const size_t fsm = sizeof(float) * (2 * dims->D_t * dims->D_t + dims->D_t * dims->rank + kFinThreads / 32);
-        if ((st = launch_pdl(lut_finalize_kernel, dim3(9, B), dim3(kFinThreads), fsm, s, f,
+        const size_t fsm = sizeof(float) * fin_smem_floats(dims->D_t, dims->rank);
+        if ((st = launch_pdl(lut_finalize_kernel, dim3(9, B), dim3(9 * B <= di.sm_count ? kFinMaxThreads : kFinMaxThreads / 2), fsm, s, f,
                              static_cast<const float *>(lut_part), static_cast<const float *>(sums_part))) != SVDLUT_OK)
             return st;
     }
@@ -1274,16 +1322,17 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
         r.dgxc = g.dg_xc;
         r.dgyc = g.dg_yc;
         r.wpart = g.dgrid_w ? wpart : nullptr;
-        // the CTA's band and strip footprint tables
-        const size_t rsm = sizeof(int) * 2 * static_cast<size_t>(pl.gp.bands + a.strips);
+        // the CTA's band and strip footprint tables, then its warps' sums
+        const size_t rsm = std::max(sizeof(int) * 2 * static_cast<size_t>(pl.gp.bands + a.strips),
+                                    sizeof(float) * (kGRThreads / 32) * dims->K);
         if (rsm > 48 * 1024) {
             if ((st = allow_dynamic_smem(reinterpret_cast<const void *>(grid_reduce_kernel), di.max_smem_optin,
                                          di.device)) != SVDLUT_OK)
                 return st;
-            if (rsm + sizeof(float) * (kGRThreads / 32) * kMaxKK > static_cast<size_t>(di.max_smem_optin))
+            if (rsm > static_cast<size_t>(di.max_smem_optin))
                 return fail(SVDLUT_ERR_UNSUPPORTED, "too many column strips and row bands for the grid reduction");
         }
-        if ((st = launch_pdl(grid_reduce_kernel, dim3(3 * (pl.sl[0] + pl.sl[1] + pl.sl[2]), B), dim3(kGRThreads), rsm, s,
+        if ((st = launch_pdl(grid_reduce_kernel, dim3(pl.sl[0] + pl.sl[1] + pl.sl[2], B), dim3(kGRThreads), rsm, s,
                              r, static_cast<const float *>(grid_part))) != SVDLUT_OK)
             return st;
         if (g.dgrid_w) {
