@@ -346,6 +346,7 @@ __global__ void __launch_bounds__(wgrad_threads(NP, SETS), wgrad_threads(NP, SET
     extern __shared__ __align__(128) char wsm[];  // stage s % 2: [A hi][A lo][B hi][B lo]
     __shared__ __align__(8) uint64_t mbar[2];
     __shared__ uint32_t taddr_s;
+    pdl_enter();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tile = blockIdx.x, z = blockIdx.y;
     const int Kd = 9 * p.Cin, P = p.So * p.So;
@@ -854,6 +855,7 @@ __global__ void __launch_bounds__(kDGT, NBUF == 2 ? 2 : (NP == 64 ? 4 : 6)) dgra
     extern __shared__ __align__(128) char dsm0[];  // stage s % NBUF: [A hi][A lo][B hi][B lo]
     __shared__ __align__(8) uint64_t mbar[2];
     __shared__ uint32_t taddr_s;
+    pdl_enter();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tile = blockIdx.x, cls = blockIdx.y, py = cls >> 1, px = cls & 1, ntx = px ? 2 : 1;
     const int Kd = (py ? 2 : 1) * ntx * p.Cout, nst = (Kd + kWK - 1) / kWK, P = p.So * p.So;
@@ -977,6 +979,7 @@ struct DPrep {
 
 __global__ void dgrad_wprep_kernel(const DPrep p)
 {
+    pdl_enter();
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < p.start[16]; e += gridDim.x * blockDim.x) {
         int g = 0;
         while (e >= p.start[g + 1]) ++g;
@@ -1138,9 +1141,7 @@ static svdlut_status launch_wgrad(const WgradArgs &a, int tiles, int chunks, cud
     constexpr int smem = 2 * wgrad_stage_bytes(NP);
     const svdlut_status st = smem_opt_in(reinterpret_cast<const void *>(wgrad_kernel<NP, SETS>), smem);
     if (st != SVDLUT_OK) return st;
-    wgrad_kernel<NP, SETS><<<dim3(tiles, chunks), wgrad_threads(NP, SETS), smem, s>>>(a);
-    SVDLUT_CUDA_TRY(cudaGetLastError());
-    return SVDLUT_OK;
+    return launch_pdl(wgrad_kernel<NP, SETS>, dim3(tiles, chunks), dim3(wgrad_threads(NP, SETS)), smem, s, a);
 }
 
 // Launch of conv_umma_kernel<NP, C8> as a programmatic dependent of the
@@ -1159,9 +1160,7 @@ static svdlut_status launch_dgrad_t(const DgradUmma &a, cudaStream_t s)
     constexpr int smem = NBUF * dgrad_stage_bytes(NP);
     const svdlut_status st = smem_opt_in(reinterpret_cast<const void *>(dgrad_umma_kernel<NP, NBUF>), smem);
     if (st != SVDLUT_OK) return st;
-    dgrad_umma_kernel<NP, NBUF><<<dim3((a.M + 127) / 128, 4), kDGT, smem, s>>>(a);
-    SVDLUT_CUDA_TRY(cudaGetLastError());
-    return SVDLUT_OK;
+    return launch_pdl(dgrad_umma_kernel<NP, NBUF>, dim3((a.M + 127) / 128, 4), dim3(kDGT), smem, s, a);
 }
 static svdlut_status launch_conv(const ConvUmma &a, int Z, cudaStream_t s)
 {
@@ -1297,42 +1296,77 @@ __device__ __forceinline__ float head_src(const ParamIn &i, int K, int h, int b,
     return *head_dst(o, K, h, b, n);
 }
 
-// dW2, db2: one thread per (h, n, j) (j = hidden unit; j = 0 also takes db2),
-// each summing over the batch in order.
-__global__ void fc2_wgrad_kernel(const float *__restrict__ hidden, ParamIn d, HeadW hw, int B, int ntot, HeadGrads hg)
+// dW2, db2: a block takes kW2Out outputs n and splits the batch over kW2Sub
+// threads each (images bs, bs + kW2Sub, ..), summed in that order; a thread
+// loads an output gradient once for all eight hidden units.  Bound by latency:
+// one chain of 64 loads per weight took 27 us at batch 64.
+constexpr int kW2Out = 32, kW2Sub = 8;
+__global__ void __launch_bounds__(kW2Out *kW2Sub)
+    fc2_wgrad_kernel(const float *__restrict__ hidden, ParamIn d, HeadW hw, int B, int ntot, HeadGrads hg)
 {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ntot * kHidden; e += gridDim.x * blockDim.x) {
-        int n = e / kHidden, h = 0;
-        const int j = e - n * kHidden;
+    pdl_enter();
+    __shared__ float part[kW2Sub][kW2Out][kHidden + 1];  // rows of 9: the lanes' stores fall in different banks
+    const int lane = threadIdx.x & 31, bs = threadIdx.x >> 5;
+    int n = blockIdx.x * kW2Out + lane, h = 0;
+    const bool in = n < ntot;
+    if (in)
         while (n >= hw.n[h]) n -= hw.n[h++];
-        float sw = 0.f, sb = 0.f;
-#pragma unroll 8
-        for (int b = 0; b < B; ++b) {  // unrolled: independent loads in flight, the same order of sums
+    float sw[kHidden] = {}, sb = 0.f;
+    if (in) {
+#pragma unroll 4
+        for (int b = bs; b < B; b += kW2Sub) {
             const float g = head_src(d, hw.K, h, b, n);
+            const float *x = hidden + b * 32 + h * 8;
             sb += g;
-            sw = fmaf(g, hidden[b * 32 + h * 8 + j], sw);
+#pragma unroll
+            for (int j = 0; j < kHidden; ++j) sw[j] = fmaf(g, x[j], sw[j]);
         }
-        if (j == 0) hg.db2[h][n] = sb;
-        hg.dw2[h][static_cast<size_t>(n) * kHidden + j] = sw;
+    }
+#pragma unroll
+    for (int j = 0; j < kHidden; ++j) part[bs][lane][j] = sw[j];
+    part[bs][lane][kHidden] = sb;
+    __syncthreads();
+    // thread (lane, bs): hidden unit bs of output lane; bs = 0 also takes db2
+    if (!in) return;
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < kW2Sub; ++q) s += part[q][lane][bs];
+    hg.dw2[h][static_cast<size_t>(n) * kHidden + bs] = s;
+    if (bs == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < kW2Sub; ++q) t += part[q][lane][kHidden];
+        hg.db2[h][n] = t;
     }
 }
+static_assert(kW2Sub == kHidden, "the sums' threads are (output, hidden unit) pairs");
 
-// dhidden[b][h][j] = sum_n dout[b][h][n] w2[h][n][j]: one CTA per (b, h).
-__global__ void __launch_bounds__(256) fc2_dgrad_kernel(ParamIn d, HeadW hw, float *__restrict__ dhid)
+// dhidden[b][h][j] = sum_n dout[b][h][n] w2[h][n][j]: one CTA per (b, h), the
+// eight sums reduced together (butterflies, then the warps in order).
+constexpr int kD2Threads = 512;
+__global__ void __launch_bounds__(kD2Threads) fc2_dgrad_kernel(ParamIn d, HeadW hw, float *__restrict__ dhid)
 {
-    __shared__ float red[8];
-    const int b = blockIdx.x, h = blockIdx.y;
+    pdl_enter();
+    __shared__ float red[kD2Threads / 32][kHidden];
+    const int b = blockIdx.x, h = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float s[kHidden] = {};
 #pragma unroll 4
-    for (int n = threadIdx.x; n < hw.n[h]; n += 256) {
+    for (int n = threadIdx.x; n < hw.n[h]; n += kD2Threads) {
         const float g = head_src(d, hw.K, h, b, n);
 #pragma unroll
         for (int j = 0; j < kHidden; ++j) s[j] = fmaf(g, hw.w2[h][static_cast<size_t>(n) * kHidden + j], s[j]);
     }
 #pragma unroll
     for (int j = 0; j < kHidden; ++j) {
-        const float t = block_sum256(s[j], red);
-        if (threadIdx.x == 0) dhid[b * 32 + h * 8 + j] = t;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
+        if (lane == 0) red[warp][j] = s[j];
+    }
+    __syncthreads();
+    if (threadIdx.x < kHidden) {
+        float t = 0.f;
+        for (int w = 0; w < kD2Threads / 32; ++w) t += red[w][threadIdx.x];
+        dhid[b * 32 + h * 8 + threadIdx.x] = t;
     }
 }
 
@@ -1340,22 +1374,25 @@ __global__ void __launch_bounds__(256) fc2_dgrad_kernel(ParamIn d, HeadW hw, flo
 __global__ void fc1_bwd_kernel(const float *__restrict__ rho, const float *__restrict__ dhid, HeadW hw, int B,
                                HeadGrads hg, float *__restrict__ drho)
 {
+    pdl_enter();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < 4 * kHidden * kRho) {
         const int h = e / (kHidden * kRho), r = e - h * kHidden * kRho, j = r / kRho, i = r - j * kRho;
-        float s = 0.f;
-        for (int b = 0; b < B; ++b) s = fmaf(dhid[b * 32 + h * 8 + j], rho[static_cast<size_t>(b) * kRho + i], s);
-        hg.dw1[h][r] = s;
-        if (i == 0) {
-            float sb = 0.f;
-            for (int b = 0; b < B; ++b) sb += dhid[b * 32 + h * 8 + j];
-            hg.db1[h][j] = sb;
+        float s = 0.f, sb = 0.f;
+#pragma unroll 8
+        for (int b = 0; b < B; ++b) {
+            const float g = dhid[b * 32 + h * 8 + j];
+            s = fmaf(g, rho[static_cast<size_t>(b) * kRho + i], s);
+            sb += g;
         }
+        hg.dw1[h][r] = s;
+        if (i == 0) hg.db1[h][j] = sb;
     }
     if (e < B * kRho) {
         const int b = e / kRho, i = e - b * kRho;
         float s = 0.f;
         for (int h = 0; h < 4; ++h)
+#pragma unroll
             for (int j = 0; j < kHidden; ++j) s = fmaf(dhid[b * 32 + h * 8 + j], hw.w1[h][j * kRho + i], s);
         drho[e] = s;
     }
@@ -1365,6 +1402,7 @@ __global__ void fc1_bwd_kernel(const float *__restrict__ rho, const float *__res
 __global__ void pool_bwd_kernel(const float *__restrict__ drho, const float *__restrict__ r4, int B, int training,
                                 uint64_t seed, float *__restrict__ dz)
 {
+    pdl_enter();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= B * 64 * 64) return;
     const int b = e / 4096, r = e - b * 4096, c = r >> 6, y = (r >> 3) & 7, x = r & 7;
@@ -1373,16 +1411,25 @@ __global__ void pool_bwd_kernel(const float *__restrict__ drho, const float *__r
 }
 
 // Sum of the partial weight gradients over chunks: one warp per output, lane
-// l adds chunks l, l + 32, ... in order, then a butterfly (a fixed order).
+// l adds chunks l, l + 32, ... in order (eight loads at a time), then a
+// butterfly (a fixed order).
 // Partials are [chunks][N][Kd + 1]; column Kd is the bias gradient.
 __global__ void wgrad_reduce_kernel(const float *__restrict__ part, int chunks, int N, int Kd, float *__restrict__ dw,
                                     float *__restrict__ db)
 {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_out = N * (Kd + 1);
     if (e >= n_out) return;  // whole warps leave together
     float s = 0.f;
-    for (int z = lane; z < chunks; z += 32) s += __ldg(part + static_cast<size_t>(z) * n_out + e);
+    for (int z0 = lane; z0 < chunks; z0 += 8 * 32) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            v[u] = z0 + 32 * u < chunks ? __ldg(part + static_cast<size_t>(z0 + 32 * u) * n_out + e) : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
@@ -1396,14 +1443,21 @@ __global__ void wgrad_reduce_kernel(const float *__restrict__ part, int chunks, 
 __global__ void __launch_bounds__(256) in_bwd_sums_kernel(const float *__restrict__ da, const float *__restrict__ r,
                                                           const float *mean, const float *rstd, int HW, float *sums)
 {
+    pdl_enter();
     __shared__ float red[8];
     const size_t o = static_cast<size_t>(blockIdx.x) * HW;
     const float mu = mean[blockIdx.x], rs = rstd[blockIdx.x];
     float s1 = 0.f, s2 = 0.f;
-    for (int i = threadIdx.x; i < HW; i += 256) {
-        const float g = da[o + i];
-        s1 = fmaf(g, (r[o + i] - mu) * rs, s1);
-        s2 += g;
+    // four elements per thread and turn (HW % 4 == 0)
+    const float4 *a4 = reinterpret_cast<const float4 *>(da + o), *r4 = reinterpret_cast<const float4 *>(r + o);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < HW / 4; i += 256) {
+        const float4 g = a4[i], x = r4[i];
+        s1 = fmaf(g.x, (x.x - mu) * rs, s1);
+        s1 = fmaf(g.y, (x.y - mu) * rs, s1);
+        s1 = fmaf(g.z, (x.z - mu) * rs, s1);
+        s1 = fmaf(g.w, (x.w - mu) * rs, s1);
+        s2 += (g.x + g.y) + (g.z + g.w);
     }
     const float t1 = block_sum256(s1, red);
     const float t2 = block_sum256(s2, red);
@@ -1414,15 +1468,38 @@ __global__ void __launch_bounds__(256) in_bwd_sums_kernel(const float *__restric
 }
 
 // pass 2: dz = LeakyReLU'(r) * rstd * gamma * (dA - s2/n - xh s1/n)
-// Four elements per thread (HW % 4 == 0: one plane per quad; float4 I/O).
+// Four elements per thread (HW % 4 == 0: one plane per quad; float4 I/O).  The
+// last CTA takes dgamma[c], dbeta[c], the sums over the batch: a warp per
+// channel, lane l adds images l, l + 32, .. in order, then a butterfly.
 __global__ void in_bwd_apply_kernel(const float *__restrict__ da, const float *__restrict__ r, const float *mean,
-                                    const float *rstd, const float *gam, const float *sums, int C, int HW, size_t n,
-                                    float *__restrict__ dz)
+                                    const float *rstd, const float *gam, const float *sums, int B, int C, int HW,
+                                    size_t n, float *__restrict__ dz, float *__restrict__ dg, float *__restrict__ db)
 {
+    pdl_enter();
+    if (blockIdx.x == gridDim.x - 1) {
+        const int lane = threadIdx.x & 31;
+        for (int c = threadIdx.x >> 5; c < C; c += blockDim.x >> 5) {
+            float a = 0.f, b2 = 0.f;
+            for (int b = lane; b < B; b += 32) {
+                a += sums[2 * (b * C + c)];
+                b2 += sums[2 * (b * C + c) + 1];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                b2 += __shfl_xor_sync(0xffffffffu, b2, o);
+            }
+            if (lane == 0) {
+                dg[c] = a;
+                db[c] = b2;
+            }
+        }
+        return;
+    }
     const float inv = 1.f / HW;
     const size_t n4 = n / 4;
     for (size_t e4 = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e4 < n4;
-         e4 += static_cast<size_t>(gridDim.x) * blockDim.x) {
+         e4 += static_cast<size_t>(gridDim.x - 1) * blockDim.x) {
         const unsigned int bc = static_cast<unsigned int>(4 * e4 / static_cast<unsigned int>(HW));
         const int c = static_cast<int>(bc % static_cast<unsigned int>(C));
         const float rs = rstd[bc], mu = mean[bc], g = rs * gam[c];
@@ -1438,20 +1515,6 @@ __global__ void in_bwd_apply_kernel(const float *__restrict__ da, const float *_
         }
         reinterpret_cast<float4 *>(dz)[e4] = make_float4(o[0], o[1], o[2], o[3]);
     }
-}
-
-// dgamma[c], dbeta[c] = sums over the batch (in order)
-__global__ void in_param_grad_kernel(const float *sums, int B, int C, float *dg, float *db)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    float a = 0.f, b2 = 0.f;
-    for (int b = 0; b < B; ++b) {
-        a += sums[2 * (b * C + c)];
-        b2 += sums[2 * (b * C + c) + 1];
-    }
-    dg[c] = a;
-    db[c] = b2;
 }
 
 __global__ void adam_kernel(float *w, const float *__restrict__ g, float *m, float *v, size_t n, float lr, float b1,
@@ -1689,11 +1752,16 @@ extern "C" svdlut_status svdlut_generator_backward(int K, const float *weights, 
     const ParamIn pin{dparams->U, dparams->S, dparams->V, dparams->lut_w, dparams->g_xy, dparams->g_xc,
                       dparams->g_yc, dparams->grid_w};
     const int ntot = L.head_n[0] + L.head_n[1] + L.head_n[2] + L.head_n[3];
-    fc2_wgrad_kernel<<<blocks_for(static_cast<size_t>(ntot) * kHidden), 256, 0, s>>>(w + wl.hidden, pin, hw, B, ntot,
-                                                                                    hg);
-    fc2_dgrad_kernel<<<dim3(B, 4), 256, 0, s>>>(pin, hw, w + wl.dhid);
-    fc1_bwd_kernel<<<(std::max(4 * kHidden * kRho, B * kRho) + 255) / 256, 256, 0, s>>>(
-        w + wl.rho, w + wl.dhid, hw, B, hg, w + wl.drho);
+    // a chain of small kernels, each a programmatic dependent launch of the one before
+    const float *hidden = w + wl.hidden;
+    if ((st = launch_pdl(fc2_wgrad_kernel, dim3((ntot + kW2Out - 1) / kW2Out), dim3(kW2Out * kW2Sub), 0, s, hidden, pin, hw, B,
+                         ntot, hg)) != SVDLUT_OK)
+        return st;
+    if ((st = launch_pdl(fc2_dgrad_kernel, dim3(B, 4), dim3(kD2Threads), 0, s, pin, hw, w + wl.dhid)) != SVDLUT_OK) return st;
+    if ((st = launch_pdl(fc1_bwd_kernel, dim3((std::max(4 * kHidden * kRho, B * kRho) + 255) / 256), dim3(256), 0, s,
+                         static_cast<const float *>(w + wl.rho), static_cast<const float *>(w + wl.dhid), hw, B, hg,
+                         w + wl.drho)) != SVDLUT_OK)
+        return st;
     {  // the input-gradient weights of layers 1..4 in the tensor cores' B layout
         DPrep dp{};
         int e = 0;
@@ -1714,11 +1782,13 @@ extern "C" svdlut_status svdlut_generator_backward(int K, const float *weights, 
             }
         }
         dp.start[16] = e;
-        dgrad_wprep_kernel<<<(e + 255) / 256, 256, 0, s>>>(dp);
+        if ((st = launch_pdl(dgrad_wprep_kernel, dim3((e + 255) / 256), dim3(256), 0, s, dp)) != SVDLUT_OK) return st;
     }
     float *dz = w + wl.dz[0];
-    pool_bwd_kernel<<<(B * 4096 + 255) / 256, 256, 0, s>>>(w + wl.drho, w + wl.r[4], B, training, seed, dz);
-    SVDLUT_CUDA_TRY(cudaGetLastError());
+    if ((st = launch_pdl(pool_bwd_kernel, dim3((B * 4096 + 255) / 256), dim3(256), 0, s,
+                         static_cast<const float *>(w + wl.drho), static_cast<const float *>(w + wl.r[4]), B, training, seed,
+                         dz)) != SVDLUT_OK)
+        return st;
     for (int i = 4; i >= 0; --i) {
         const int Cin = kCh[i], Cout = kCh[i + 1], S = kSz[i], So = kSz[i + 1];
         const int pix = B * So * So, Kd = Cin * 9, chunk = wgrad_chunk_px(B, i), chunks = wgrad_chunks(B, i);
@@ -1733,9 +1803,10 @@ extern "C" svdlut_status svdlut_generator_backward(int K, const float *weights, 
             st = np == 16 ? launch_wgrad<16, 1>(wa, tiles, chunks, s)
                           : np == 32 ? launch_wgrad<32, 1>(wa, tiles, chunks, s) : launch_wgrad<64, 1>(wa, tiles, chunks, s);
         if (st != SVDLUT_OK) return st;
-        wgrad_reduce_kernel<<<(Cout * (Kd + 1) * 32 + 255) / 256, 256, 0, s>>>(
-            w + wl.wpart, chunks * sets, Cout, Kd, dweights + L.conv_w[i], dweights + L.conv_b[i]);
-        SVDLUT_CUDA_TRY(cudaGetLastError());
+        if ((st = launch_pdl(wgrad_reduce_kernel, dim3((Cout * (Kd + 1) * 32 + 255) / 256), dim3(256), 0, s,
+                             static_cast<const float *>(w + wl.wpart), chunks * sets, Cout, Kd, dweights + L.conv_w[i],
+                             dweights + L.conv_b[i])) != SVDLUT_OK)
+            return st;
         if (i == 0) break;
         // input gradient, then InstanceNorm + LeakyReLU backward of layer i-1
         float *dact = w + wl.dact;
@@ -1755,13 +1826,15 @@ extern "C" svdlut_status svdlut_generator_backward(int K, const float *weights, 
         }
         const int j = i - 1;
         float *dz_next = dz == w + wl.dz[0] ? w + wl.dz[1] : w + wl.dz[0];
-        in_bwd_sums_kernel<<<B * Cin, 256, 0, s>>>(dact, w + wl.r[j], w + wl.mean[j], w + wl.rstd[j], S * S,
-                                                   w + wl.insum);
+        const float *da = dact, *rj = w + wl.r[j], *mean = w + wl.mean[j], *rstd = w + wl.rstd[j], *sums = w + wl.insum;
+        if ((st = launch_pdl(in_bwd_sums_kernel, dim3(B * Cin), dim3(256), 0, s, da, rj, mean, rstd, S * S, w + wl.insum)) !=
+            SVDLUT_OK)
+            return st;
         const size_t n = act_size(B, j);
-        in_bwd_apply_kernel<<<blocks_for(n / 4), 256, 0, s>>>(dact, w + wl.r[j], w + wl.mean[j], w + wl.rstd[j],
-                                                          weights + L.in_g[j], w + wl.insum, Cin, S * S, n, dz_next);
-        in_param_grad_kernel<<<1, 64, 0, s>>>(w + wl.insum, B, Cin, dweights + L.in_g[j], dweights + L.in_b[j]);
-        SVDLUT_CUDA_TRY(cudaGetLastError());
+        if ((st = launch_pdl(in_bwd_apply_kernel, dim3(blocks_for(n / 4) + 1), dim3(256), 0, s, da, rj, mean, rstd,
+                             weights + L.in_g[j], sums, B, Cin, S * S, n, dz_next, dweights + L.in_g[j],
+                             dweights + L.in_b[j])) != SVDLUT_OK)
+            return st;
         dz = dz_next;
     }
     return SVDLUT_OK;
