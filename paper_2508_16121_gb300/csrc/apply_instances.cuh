@@ -10,9 +10,9 @@ namespace svdlut {
 
 // Launches one instance as a dependent of the preceding kernel (prep_kernel, or
 // any other): it may be launched while that one runs, and waits for it before
-// it reads anything (with PRE, before it reads the tables: prep_kernel has
-// waited for what came before).
-template <class IO, int N, bool DX, bool PRE, bool FAST>
+// it reads anything (after prep_kernel, before it reads the tables: prep_kernel
+// has waited for what came before).
+template <class IO, int N, bool DX, int PRE, bool FAST>
 svdlut_status launch_instance(LaunchArgs<N> &a, size_t smem, const DeviceInfo &di, cudaStream_t s, int grid)
 {
     svdlut_status st = allow_smem_once(reinterpret_cast<const void *>(apply_kernel<IO, N, DX, PRE, FAST>),
@@ -27,11 +27,14 @@ svdlut_status launch_instance(LaunchArgs<N> &a, size_t smem, const DeviceInfo &d
 template <class IO, int N, bool DX>
 svdlut_status launch_io(LaunchArgs<N> &a, size_t smem, const DeviceInfo &di, cudaStream_t s, int grid)
 {
-    if (a.pre) return launch_instance<IO, N, DX, true, false>(a, smem, di, s, grid);
-    bool fast = a.xcol != 0;
-    for (int i = 0; i < a.n; ++i) fast = fast && fast_rows(a.img[i]);
-    return fast ? launch_instance<IO, N, DX, false, true>(a, smem, di, s, grid)
-                : launch_instance<IO, N, DX, false, false>(a, smem, di, s, grid);
+    if constexpr (!DX)
+        if (a.pre == kPreFolds) return launch_instance<IO, N, DX, kPreFolds, true>(a, smem, di, s, grid);
+    const bool fast = all_fast_rows(a);
+    if constexpr (std::is_same<IO, IoF32>::value && !DX)  // 1 % at most; none with 8-bit pixels
+        if (a.pre && fast) return launch_instance<IO, N, DX, kPreAll, true>(a, smem, di, s, grid);
+    if (a.pre) return launch_instance<IO, N, DX, kPreAll, false>(a, smem, di, s, grid);
+    return fast ? launch_instance<IO, N, DX, kPreNone, true>(a, smem, di, s, grid)
+                : launch_instance<IO, N, DX, kPreNone, false>(a, smem, di, s, grid);
 }
 
 }  // namespace svdlut

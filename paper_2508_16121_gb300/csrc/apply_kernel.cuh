@@ -63,6 +63,10 @@ struct ImgDesc {
                    // yc [3][Dsy][Dsc], then the three summed biases
 };
 
+// Precomputed by prep_kernel: nothing, the cell tables and the folded grids, or
+// the folded grids alone.
+enum { kPreNone = 0, kPreAll = 1, kPreFolds = 2 };
+
 template <int N>
 struct LaunchArgs {
     int n;             // images in img[]
@@ -71,7 +75,7 @@ struct LaunchArgs {
     int lcell_floats;    // floats reserved for the cell table
     int scratch_floats;  // floats of the block buffers / prologue temporaries
     int xcol;            // nonzero: per-column xc tables (every image's Dsc <= kXcolMaxDsc)
-    int pre;             // nonzero: cell tables and folded grids precomputed (the PRE kernel)
+    int pre;             // what prep_kernel has precomputed: kPreNone, kPreAll or kPreFolds
     unsigned int *queue;  // non-null: blocks are taken from this counter (must be 0 at launch)
     unsigned int *check;  // index-check status (builds with SVDLUT_CHECK_BOUNDS), else null
     ImgDesc img[N];
@@ -1011,6 +1015,7 @@ constexpr int kPrepThreads = 512;
 template <int N>
 struct PrepArgs {
     int n;
+    int lut_ctas;      // CTAs per image that build cell tables: kLutCtas, or 0
     int start[N + 1];  // first fold output of each image in the flat index (host prefix sums)
     ImgDesc img[N];
 };
@@ -1031,7 +1036,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const __grid_constan
     asm volatile("griddepcontrol.launch_dependents;\n" :::);
     extern __shared__ __align__(16) float ps[];
     const int tid = threadIdx.x;
-    if (static_cast<int>(blockIdx.x) < kLutCtas * a.n) {
+    if (static_cast<int>(blockIdx.x) < a.lut_ctas * a.n) {
         const ImgDesc &d = a.img[blockIdx.x / kLutCtas];
         const int rem = blockIdx.x % kLutCtas, p = rem / kLutParts, part = rem - p * kLutParts;
         const int D = d.D, R = d.R, Rp = padded_rank(R), R4 = (R + 3) / 4, DR = D * R, DRp = D * Rp, Dm1 = D - 1;
@@ -1104,9 +1109,9 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const __grid_constan
     // loads of kBatch outputs are issued before their sums); image i owns the
     // flat outputs [start[i], start[i + 1])
     const int total = a.start[a.n];
-    const int stride = (static_cast<int>(gridDim.x) - kLutCtas * a.n) * kPrepThreads;
+    const int stride = (static_cast<int>(gridDim.x) - a.lut_ctas * a.n) * kPrepThreads;
     constexpr int kBatch = 4, kTerms = 3;
-    for (int t0 = (static_cast<int>(blockIdx.x) - kLutCtas * a.n) * kPrepThreads + tid; t0 < total;
+    for (int t0 = (static_cast<int>(blockIdx.x) - a.lut_ctas * a.n) * kPrepThreads + tid; t0 < total;
          t0 += kBatch * stride) {
         float g[kBatch][kTerms], w[kBatch][kTerms];
         int which[kBatch], ch[kBatch], im[kBatch], o[kBatch], e[kBatch];
@@ -1298,13 +1303,16 @@ __host__ __device__ __forceinline__ bool fast_rows(const ImgDesc &d)
 // plane).  Every pixel gathers its own cells: reusing a lane's previous cell
 // when unchanged saved shared-memory wavefronts in smooth regions but cost
 // more in compares than it saved.
-// PRE: cell tables and folded grids come from prep_kernel (ImgDesc::pcell,
-// pfold); otherwise every CTA builds them.  FAST: every image takes fast rows;
-// otherwise each block decides.  Both are template parameters because the
-// pixel loop needs all 128 registers: with the table construction and the
-// general rows in the same kernel it spilled, and 4K frames took 100 us
-// instead of 94 (PRE alone is small enough for both kinds of rows).
-template <class IO, int N, bool DX, bool PRE, bool FAST>
+// PRE: what comes from prep_kernel (ImgDesc::pcell, pfold): everything, only
+// the folded grids, or nothing; a CTA builds the rest.  kPreFolds: the CTA copies
+// the factors and builds the cells while prep_kernel folds the grids, instead of
+// copying 152 KB of cells after it; it wants what copy_factors and fast rows want
+// from every image.  FAST: every image takes fast rows; otherwise each block
+// decides.  Both are template parameters because the pixel loop needs all 128
+// registers: with the table construction and the general rows in the same
+// kernel it spilled, and 4K frames took 100 us instead of 94 (kPreAll alone is
+// small enough for both kinds of rows).
+template <class IO, int N, bool DX, int PRE, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constant__ LaunchArgs<N> a)
 {
     extern __shared__ __align__(16) float smem[];
@@ -1315,7 +1323,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
     // the next kernel of the stream (e.g. the next call's prep_kernel, which
     // waits for this one before reading anything) may begin launching
     asm volatile("griddepcontrol.launch_dependents;\n" :::);
-    if constexpr (!PRE) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if constexpr (PRE == kPreNone) asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool xcol = FAST || a.xcol != 0;
     // Block schedule: a contiguous range per CTA, or (queue) blocks taken in
@@ -1381,7 +1389,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
 
     Raw cur[NP], nxt[NP];
     int cur_im = -1;
-    bool first = true, pre_wait = PRE;
+    bool first = true, pre_wait = PRE != kPreNone;
     for (;;) {
         const int im = find_image(blk);
         const ImgDesc &d = a.img[im];
@@ -1396,7 +1404,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
             }
         };
         __syncthreads();  // previous block's rows done with the buffers and the cell table
-        if constexpr (PRE) {
+        if constexpr (PRE == kPreAll) {
             // The pixels are inputs of the call, complete before the launch:
             // the first row is requested while the precomputation may still
             // run (programmatic dependent launch); the tables after it ends.
@@ -1409,10 +1417,28 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
             cp_async_wait_all();
             __syncthreads();
         }
+        if constexpr (PRE == kPreFolds) {
+            // pixels and factors are inputs of the call, complete before the
+            // launch; the folded grids come after the wait for prep_kernel
+            if (im != cur_im) {
+                copy_factors(d, b.xcol, misc);
+                cp_async_wait_all();
+                __syncthreads();
+                build_cells(d.D, b.xcol, lcell);
+            }
+            first_row();
+            if (pre_wait) {
+                asm volatile("griddepcontrol.wait;\n" ::: "memory");
+                pre_wait = false;
+            }
+            setup_pre(d, g, b, lcell, misc, false);
+            cp_async_wait_all();
+            __syncthreads();
+        }
         // the factors' place: the block buffers from the xc slice on
-        const bool overlap = !PRE && im != cur_im && fast_factors_ok(d) &&
+        const bool overlap = PRE == kPreNone && im != cur_im && fast_factors_ok(d) &&
                              (b.xcol - scratch) + fast_factor_floats(d.D) <= a.scratch_floats;
-        if constexpr (!PRE) {
+        if constexpr (PRE == kPreNone) {
             if (overlap) {
                 copy_factors(d, b.xcol, misc);
             } else if (im != cur_im) {
@@ -1423,8 +1449,8 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
         cur_im = im;
         first_row();
         if (a.queue && threadIdx.x == 0) *slot = static_cast<int>(atomicAdd(a.queue, 1u));
-        block_phase_a<!PRE>(d, g, b);
-        if constexpr (!PRE) {
+        block_phase_a<PRE == kPreNone>(d, g, b);
+        if constexpr (PRE == kPreNone) {
             if (overlap) {
                 cp_async_wait_all();
                 __syncthreads();

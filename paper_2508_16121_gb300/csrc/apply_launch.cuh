@@ -138,10 +138,11 @@ inline void set_prep_tables(ImgDesc &e, const svdlut_dims *d, char *w)
 }
 
 template <int N>
-svdlut_status launch_prep(const LaunchArgs<N> &a, int sm_count, cudaStream_t s)
+svdlut_status launch_prep(const LaunchArgs<N> &a, int sm_count, cudaStream_t s, bool luts = true)
 {
     PrepArgs<N> pa{};
     pa.n = a.n;
+    pa.lut_ctas = luts ? kLutCtas : 0;
     double total = 0;
     int smem_fl = 0;
     for (int i = 0; i < a.n; ++i) {
@@ -154,34 +155,57 @@ svdlut_status launch_prep(const LaunchArgs<N> &a, int sm_count, cudaStream_t s)
         smem_fl = std::max(smem_fl, prep_smem_floats(e.D, e.R));
     }
     pa.start[a.n] = static_cast<int>(total);
-    const int fold_ctas = std::max(sm_count, 2 * sm_count - kLutCtas * a.n);
+    const int fold_ctas = std::max(sm_count, 2 * sm_count - pa.lut_ctas * a.n);
     const size_t smem = sizeof(float) * static_cast<size_t>(smem_fl);
     // programmatic dependent of the preceding kernel (it waits for it first)
-    return launch_pdl(prep_kernel<N>, dim3(kLutCtas * a.n + fold_ctas), dim3(kPrepThreads), smem, s, pa);
+    return launch_pdl(prep_kernel<N>, dim3(pa.lut_ctas * a.n + fold_ctas), dim3(kPrepThreads), smem, s, pa);
 }
 
-// Whether the precomputed tables are worth their launch for planned args on
-// `ctas` CTAs.  Without them a CTA folds its blocks' raw grids itself, K times
-// the loads of the folded slices; that takes longer from about 9000 loads a
-// CTA on, while the launch of prep_kernel and the wait for it cost about 4 us
-// whatever the size: 64 images of 256 x 256 with 17-vertex grids (5 K loads)
-// take 84 us without and 91 with, 16 of 480 x 640 with grids at 1/8 resolution
-// (12 K) 92 and 92, a 4K frame (18 K) 99 and 95.  Only the factors that
-// copy_factors takes are built quickly in the CTAs.
+// Whether every image takes fast rows.
 template <int N>
-bool tables_pay(const LaunchArgs<N> &a, int ctas)
+bool all_fast_rows(const LaunchArgs<N> &a)
 {
-    constexpr double kMaxLoads = 9216;
-    double loads = 0;
+    bool fast = a.xcol != 0;
+    for (int i = 0; i < a.n; ++i) fast = fast && fast_rows(a.img[i]);
+    return fast;
+}
+
+// Whether every image's factors are taken by copy_factors and fit the place
+// that the kernel gives them (the block buffers from the xc slice on).
+template <int N>
+bool factors_in_ctas(const LaunchArgs<N> &a)
+{
     for (int i = 0; i < a.n; ++i) {
         const ImgDesc &e = a.img[i];
         const int nvx = span_bound(kTileW, e.W, e.Dsx), nvy = span_bound(e.BH, e.H, e.Dsy);
         const int xcol = fold_floats(nvx, nvy, e.Dsc) + 2 * kTileW + ((2 * a.bh_max + 3) & ~3);
-        if (!fast_factors_ok(e) || xcol + fast_factor_floats(e.D) > a.scratch_floats) return true;
-        const int blocks = (i + 1 < a.n ? a.img[i + 1].block_begin : a.total_blocks) - e.block_begin;
-        loads += static_cast<double>(blocks) * e.K * (nvx * nvy + (nvx + nvy) * e.Dsc);
+        if (!fast_factors_ok(e) || xcol + fast_factor_floats(e.D) > a.scratch_floats) return false;
     }
-    return loads > kMaxLoads * std::min(ctas, a.total_blocks);
+    return true;
+}
+
+// Launches prep_kernel for planned args where it pays and sets a.pre.  Device
+// times of one launch with everything built in the CTAs / everything from
+// prep_kernel / the folded grids from prep_kernel, us:
+//   1 x 64x64     12.7 / 10.1 / 12.1    16 x 256x256  27.7 / 28.0 / 28.3
+//   1 x 853x1279  27.6 / 26.1 / 27.3    30 x 256x256  45.9 / 47.9 / 46.3
+//   1 x 4K        99.4 / 94.9 / 98.0    64 x 256x256  84.4 / 90.2 / 84.5
+//   4 x 1080p u8  99.1 / 97.2 / 98.4    77 x 190x558 u8  249 / 262 / 238
+// Few images: all CTAs copy one table while a few build it.  From kManyImages
+// on the tables cost as much as they save, the folds still pay.  Up to
+// kLaunchBoundPx pixels the call is bound by its launches (20 us of host time
+// with one, 23 with two), so it makes one.
+constexpr int kManyImages = 16;
+constexpr double kLaunchBoundPx = 512.0 * 1024.0;
+template <int N>
+svdlut_status launch_tables(LaunchArgs<N> &a, int sm_count, cudaStream_t s)
+{
+    double px = 0;
+    for (int i = 0; i < a.n; ++i) px += static_cast<double>(a.img[i].H) * a.img[i].W;
+    const bool in_ctas = factors_in_ctas(a);
+    if (in_ctas && px <= kLaunchBoundPx) return SVDLUT_OK;
+    a.pre = in_ctas && a.n >= kManyImages && all_fast_rows(a) ? kPreFolds : kPreAll;
+    return launch_prep(a, sm_count, s, a.pre == kPreAll);
 }
 
 // Launches apply_kernel for args whose blocks are already planned.  dx_mode

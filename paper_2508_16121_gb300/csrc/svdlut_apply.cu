@@ -134,10 +134,7 @@ static svdlut_status apply_chunks(const svdlut_dims *dims, const svdlut_params *
         size_t smem = 0;
         if ((st = plan_uniform(a, n_cta, static_cast<size_t>(di.max_smem_optin), &smem)) != SVDLUT_OK)
             return st;
-        if (ws && tables_pay(a, n_cta)) {
-            if ((st = launch_prep(a, di.sm_count, s)) != SVDLUT_OK) return st;
-            a.pre = 1;
-        }
+        if (ws && (st = launch_tables(a, di.sm_count, s)) != SVDLUT_OK) return st;
         if ((st = launch_apply(a, smem, dtype, s, n_cta)) != SVDLUT_OK) return st;
     }
     return SVDLUT_OK;

@@ -1174,7 +1174,7 @@ static svdlut_status dx_chunks(const svdlut_dims *dims, const svdlut_params *par
         if ((st = plan_uniform(a, di.sm_count, static_cast<size_t>(di.max_smem_optin), &smem)) != SVDLUT_OK) return st;
         if (tables) {
             if ((st = launch_prep(a, di.sm_count, s)) != SVDLUT_OK) return st;
-            a.pre = 1;
+            a.pre = kPreAll;
         }
         if ((st = launch_apply(a, smem, SVDLUT_F32, s, 0, true)) != SVDLUT_OK) return st;
     }

@@ -133,10 +133,7 @@ static svdlut_status run_batched(const svdlut_image *imgs, int n, svdlut_dtype d
                 set_prep_tables(a.img[i], &imgs[i0 + i].dims, tab);
                 tab += prep_image_bytes(&imgs[i0 + i].dims);
             }
-            if (tables_pay(a, ctas)) {
-                if ((st = launch_prep(a, di.sm_count, s)) != SVDLUT_OK) return st;
-                a.pre = 1;
-            }
+            if ((st = launch_tables(a, di.sm_count, s)) != SVDLUT_OK) return st;
         }
         if ((st = launch_apply(a, smem, dtype, s, std::min(ctas, a.total_blocks))) != SVDLUT_OK) return st;
     }
