@@ -196,12 +196,27 @@ constexpr int kMiscFloats = kMaxK * 4 + 4;
 template <typename T>
 struct PixIO;
 
+// Whole lanes (n = 4) of an unaligned row take the widest accesses that its
+// address allows: lanes are 16 bytes apart, so a warp-wide 4-byte access is 4
+// passes of the shared-memory pipe, as is a 16-byte one, and the rows of an
+// image of odd width are at every offset in turn: 9 passes a plane on average
+// (6 for even widths) where four 4-byte accesses are 16.
 template <>
 struct PixIO<float> {
     using Raw = float4;
     static __device__ __forceinline__ Raw load(const float *p, int n, bool vec)
     {
         if (vec && n == 4) return __ldcs(reinterpret_cast<const float4 *>(p));
+        if (n == 4) {
+            const unsigned int word = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(p) >> 2) & 3u;
+            if (word == 0u) return __ldcs(reinterpret_cast<const float4 *>(p));
+            if (word == 2u) {
+                const float2 a = __ldcs(reinterpret_cast<const float2 *>(p)), b = __ldcs(reinterpret_cast<const float2 *>(p + 2));
+                return make_float4(a.x, a.y, b.x, b.y);
+            }
+            const float2 m = __ldcs(reinterpret_cast<const float2 *>(p + 1));
+            return make_float4(__ldcs(p), m.x, m.y, __ldcs(p + 3));
+        }
         Raw v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (n > 0) v.x = __ldcs(p);
         if (n > 1) v.y = __ldcs(p + 1);
@@ -210,27 +225,24 @@ struct PixIO<float> {
         return v;
     }
     static __device__ __forceinline__ float4 to_float(Raw v) { return v; }
-    // pixel k of a lane at p + 32 k (k < n): one coalesced 128-byte row per warp instruction
-    static __device__ __forceinline__ Raw load_s(const float *p, int n)
-    {
-        Raw v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n > 0) v.x = __ldcs(p);
-        if (n > 1) v.y = __ldcs(p + 32);
-        if (n > 2) v.z = __ldcs(p + 64);
-        if (n > 3) v.w = __ldcs(p + 96);
-        return v;
-    }
-    static __device__ __forceinline__ void store_s(float *p, float4 v, int n)
-    {
-        if (n > 0) __stcs(p, v.x);
-        if (n > 1) __stcs(p + 32, v.y);
-        if (n > 2) __stcs(p + 64, v.z);
-        if (n > 3) __stcs(p + 96, v.w);
-    }
     static __device__ __forceinline__ void store(float *p, float4 v, int n, bool vec)
     {
         if (vec && n == 4) {
             __stcs(reinterpret_cast<float4 *>(p), v);
+            return;
+        }
+        if (n == 4) {
+            const unsigned int word = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(p) >> 2) & 3u;
+            if (word == 0u) {
+                __stcs(reinterpret_cast<float4 *>(p), v);
+            } else if (word == 2u) {
+                __stcs(reinterpret_cast<float2 *>(p), make_float2(v.x, v.y));
+                __stcs(reinterpret_cast<float2 *>(p + 2), make_float2(v.z, v.w));
+            } else {
+                __stcs(p, v.x);
+                __stcs(reinterpret_cast<float2 *>(p + 1), make_float2(v.y, v.z));
+                __stcs(p + 3, v.w);
+            }
             return;
         }
         if (n > 0) __stcs(p, v.x);
@@ -1312,7 +1324,9 @@ __host__ __device__ __forceinline__ bool fast_rows(const ImgDesc &d)
 // registers: with the table construction and the general rows in the same
 // kernel it spilled, and 4K frames took 100 us instead of 94 (kPreAll alone is
 // small enough for both kinds of rows).
-template <class IO, int N, bool DX, int PRE, bool FAST>
+// VEC: every image allows whole-lane vector accesses (ImgDesc::vec); the code of
+// the unaligned ones costs the aligned frames 1.5 %.
+template <class IO, int N, bool DX, int PRE, bool FAST, bool VEC>
 __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constant__ LaunchArgs<N> a)
 {
     extern __shared__ __align__(16) float smem[];
@@ -1363,14 +1377,14 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
         const int nc = n > 0 ? checked_run(a.check, off, n, plane) : 0;
         if (nc > 0) {
             const void *px = In::at(d.x, off);
-            In::load(px, plane, nc, checked_vec(a.check, d.vec, px, In::kVecAlign), dst);
+            In::load(px, plane, nc, checked_vec(a.check, VEC || d.vec, px, In::kVecAlign), dst);
         } else {
 #pragma unroll
             for (int c = 0; c < 3; ++c) dst[c] = Raw();
         }
         if constexpr (DX) {
             const float *g = d.dy + off;
-            const bool v = checked_vec(a.check, d.vec, g, 16);
+            const bool v = checked_vec(a.check, VEC || d.vec, g, 16);
 #pragma unroll
             for (int c = 0; c < 3; ++c) dst[3 + c] = nc > 0 ? PixIO<float>::load(g + c * plane, nc, v) : Raw();
         }
@@ -1669,10 +1683,10 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                 if (nc > 0) {
                     if constexpr (!DX) {
                         const void *py = Out::at(d.y, off);
-                        Out::store(d.y, plane, off, out, nc, checked_vec(a.check, d.vec, py, Out::kVecAlign));
+                        Out::store(d.y, plane, off, out, nc, checked_vec(a.check, VEC || d.vec, py, Out::kVecAlign));
                     } else {
                         float *py = static_cast<float *>(d.y) + off;
-                        const bool v = checked_vec(a.check, d.vec, py, 16);
+                        const bool v = checked_vec(a.check, VEC || d.vec, py, 16);
 #pragma unroll
                         for (int c = 0; c < 3; ++c)
                             PixIO<float>::store(py + c * plane, make_float4(out[c][0], out[c][1], out[c][2], out[c][3]),
