@@ -180,15 +180,56 @@ inline WsLayout make_ws(int B)
 
 // ---------------------------------------------------------------- kernels
 
-// Bilinear downsample to 256x256 with half-pixel centres, no antialiasing.
-__global__ void downsample_kernel(const float *__restrict__ x, int B, int H, int W, float *__restrict__ t)
+// The five convolutions' weights as BF16 in the B stage layout of
+// conv_umma_kernel: element (o, k) of layer i at bf16 index (k / 8) * 8 NP +
+// 8 o + k % 8 for k < Kpad (whole 64-k stages), zero for o >= Cout or k >= Kd;
+// k in the kernel's reduction order ((tap, c) when Cin is a power of two >= 8,
+// else (c, tap)).
+struct WPrep {
+    const float *w[5];
+    __nv_bfloat16 *out[5];
+    int start[6];  // flattened element ranges per layer
+    int cin[5], cout[5], np[5], kpad[5];
+};
+
+__device__ __forceinline__ void prepare_conv_weight(const WPrep &p, int e)
+{
+    int i = 0;
+    while (e >= p.start[i + 1]) ++i;
+    const int Cin = p.cin[i], Cout = p.cout[i], Kd = 9 * Cin, NP = p.np[i];
+    const int l = e - p.start[i], o = l / p.kpad[i], k = l - o * p.kpad[i];
+    float v = 0.f;
+    if (o < Cout && k < Kd) {
+        int c, tap;
+        if (Cin >= 8 && (Cin & (Cin - 1)) == 0) {
+            tap = k / Cin;
+            c = k - tap * Cin;
+        } else {
+            c = k / 9;
+            tap = k - 9 * c;
+        }
+        v = p.w[i][(static_cast<size_t>(o) * Cin + c) * 9 + tap];
+    }
+    p.out[i][(k >> 3) * 8 * NP + 8 * o + (k & 7)] = __float2bfloat16_rn(v);
+}
+
+// Bilinear downsample to 256x256 with half-pixel centres, no antialiasing (CTAs
+// below nds); the CTAs after those lay out the convolutions' weights, which the
+// next kernel waits for as well.
+__global__ void downsample_kernel(const float *__restrict__ x, int B, int H, int W, float *__restrict__ t, int nds,
+                                  const WPrep wp)
 {
     static_assert(kThumb % 4 == 0, "four outputs of one thumbnail row per thread");
-    pdl_enter();
+    pdl_enter();  // the outputs may still be read by the previous call's kernels
+    if (static_cast<int>(blockIdx.x) >= nds) {
+        const int e = (static_cast<int>(blockIdx.x) - nds) * static_cast<int>(blockDim.x) + static_cast<int>(threadIdx.x);
+        if (e < wp.start[5]) prepare_conv_weight(wp, e);
+        return;
+    }
     const size_t n4 = static_cast<size_t>(B) * 3 * kThumb * kThumb / 4;
     const float sy_ = static_cast<float>(H) / kThumb, sx_ = static_cast<float>(W) / kThumb;
     for (size_t e4 = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e4 < n4;
-         e4 += static_cast<size_t>(gridDim.x) * blockDim.x) {
+         e4 += static_cast<size_t>(nds) * blockDim.x) {
         const size_t e = 4 * e4;
         const int ox0 = static_cast<int>(e % kThumb), oy = static_cast<int>((e / kThumb) % kThumb);
         const size_t bc = e / (kThumb * kThumb);
@@ -538,7 +579,7 @@ __global__ void __launch_bounds__(wgrad_threads(NP, SETS), wgrad_threads(NP, SET
 // K-major layout of wgrad_kernel: element (m, k) of a stage of kWK = 64 k at
 // byte (k / 8) * 16 * 128 + 16 m + 2 (k % 8), so a thread writes the 8 k of
 // one octet of its pixel as one 16-byte store (conflict-free across a warp's
-// consecutive pixels).  conv_wprep_kernel lays the weights out once per call
+// consecutive pixels).  downsample_kernel lays the weights out once per call
 // in exactly the stage layout of B (element (o, k) at byte (k / 8) * 16 NP +
 // 16 o + 2 (k % 8), zero for o >= Cout and k >= Kd), so a stage of B is a
 // contiguous copy.  CTA (tile, z) takes the stages [z ks, (z + 1) ks) and
@@ -557,7 +598,7 @@ __device__ __forceinline__ float warp_total(float v)
 struct ConvUmma {
     const float *in;       // [B][Cin][S][S]
     const float *sc, *sh;  // [B][Cin] affine map of the input (zero padding after it), or null
-    const uint4 *wb;       // BF16 weights in the stage layout (conv_wprep_kernel)
+    const uint4 *wb;       // BF16 weights in the stage layout (downsample_kernel)
     float *part;           // [Z][Cout][M]
     int Cin, S, So, Cout, M, Kd, ks;  // ks: stages of 64 k per split
     // fused finish (one split, So^2 a multiple of 128, r set): the epilogue
@@ -776,42 +817,6 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 8 : (NP == 64 ? 2 : 3)) conv_u
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;\n");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(kCols));
-    }
-}
-
-// The five convolutions' weights as BF16 in the B stage layout of
-// conv_umma_kernel: element (o, k) of layer i at bf16 index (k / 8) * 8 NP +
-// 8 o + k % 8 for k < Kpad (whole 64-k stages), zero for o >= Cout or k >= Kd;
-// k in the kernel's reduction order ((tap, c) when Cin is a power of two >= 8,
-// else (c, tap)).
-struct WPrep {
-    const float *w[5];
-    __nv_bfloat16 *out[5];
-    int start[6];  // flattened element ranges per layer
-    int cin[5], cout[5], np[5], kpad[5];
-};
-
-__global__ void conv_wprep_kernel(const WPrep p)
-{
-    pdl_enter();  // the outputs may still be read by the previous call's kernels
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < p.start[5]; e += gridDim.x * blockDim.x) {
-        int i = 0;
-        while (e >= p.start[i + 1]) ++i;
-        const int Cin = p.cin[i], Cout = p.cout[i], Kd = 9 * Cin, NP = p.np[i];
-        const int l = e - p.start[i], o = l / p.kpad[i], k = l - o * p.kpad[i];
-        float v = 0.f;
-        if (o < Cout && k < Kd) {
-            int c, tap;
-            if (Cin >= 8 && (Cin & (Cin - 1)) == 0) {
-                tap = k / Cin;
-                c = k - tap * Cin;
-            } else {
-                c = k / 9;
-                tap = k - 9 * c;
-            }
-            v = p.w[i][(static_cast<size_t>(o) * Cin + c) * 9 + tap];
-        }
-        p.out[i][(k >> 3) * 8 * NP + 8 * o + (k & 7)] = __float2bfloat16_rn(v);
     }
 }
 
@@ -1661,10 +1666,7 @@ extern "C" svdlut_status svdlut_generator_forward(int K, const float *weights, i
     const WsLayout wl = make_ws(B);
     float *w = static_cast<float *>(ws);
     // a chain of small kernels, each a programmatic dependent launch of the one before
-    if ((st = launch_pdl(downsample_kernel, dim3(static_cast<int>((static_cast<size_t>(B) * 3 * kThumb * kThumb / 4 + 255) / 256)),
-                         dim3(256), 0, s, x, B, H, W, w + wl.thumb)) != SVDLUT_OK)
-        return st;
-    {  // the convolutions' weights in the tensor cores' B layout
+    {  // the thumbnail, and the convolutions' weights in the tensor cores' B layout
         WPrep wp{};
         int e = 0;
         for (int i = 0; i < 5; ++i) {
@@ -1678,7 +1680,10 @@ extern "C" svdlut_status svdlut_generator_forward(int K, const float *weights, i
             e += static_cast<int>(conv_wbf_elems(i));
         }
         wp.start[5] = e;
-        if ((st = launch_pdl(conv_wprep_kernel, dim3((e + 255) / 256), dim3(256), 0, s, wp)) != SVDLUT_OK) return st;
+        const int nds = static_cast<int>((static_cast<size_t>(B) * 3 * kThumb * kThumb / 4 + 255) / 256);
+        if ((st = launch_pdl(downsample_kernel, dim3(nds + (e + 255) / 256), dim3(256), 0, s, x, B, H, W, w + wl.thumb, nds,
+                             wp)) != SVDLUT_OK)
+            return st;
     }
     const float *in = w + wl.thumb, *isc = nullptr, *ish = nullptr;
     for (int i = 0; i < 5; ++i) {
