@@ -3,11 +3,9 @@
 // One persistent CTA per SM walks a contiguous range of pixel blocks (or takes
 // blocks from an atomic queue, for ragged batches); a block is a
 // 128-pixel-wide column strip of one image, BH rows tall (BH is planned on the
-// host so that the blocks cover the SMs evenly).  A lane owns 4 pixels of a
-// row: columns lane + 32 k of the tile for float images (every warp-wide
-// access covers 32 adjacent pixels, which keeps the table gathers of smooth
-// regions on few cells), or 4 adjacent pixels for integer pixel formats (one
-// 32- or 64-bit access per plane or word); warp w owns rows w, w + kWarps, ...
+// host so that the blocks cover the SMs evenly).  A lane owns 4 adjacent pixels
+// of a row (one 128-bit access per float plane where the row is aligned, one 32-
+// or 64-bit access per integer plane or word); warp w owns rows w, w + kWarps, ...
 // of the block.  The pixel formats (planar float and 8-bit, interleaved
 // 8-bit) are template parameters (Io<In, Out> below).
 //  - Prologue, once per image a CTA meets: the factor rows arrive by
