@@ -680,7 +680,8 @@ __global__ void __launch_bounds__(kGridThreads, 1)
 // LUT finalize: one CTA per (table c*3+pair, image).  The image's partials are
 // summed in up to kFinParts contiguous parts, side by side, kFinBatch loads at a
 // time, then the parts in order: two images' 152 partials on 18 CTAs were bound
-// by the latency of one chain of loads per vertex (76 us at 2 x 342x628).
+// by the latency of one chain of loads per vertex (76 us at 2 x 342x628; 17 us at
+// 8 x 1920x1080 and at 64 x 256x256 as it is, 27 and 20 before).
 // ---------------------------------------------------------------------------
 constexpr int kFinMaxThreads = 1024, kFinParts = 8, kFinBatch = 8;
 
@@ -796,7 +797,7 @@ __global__ void __launch_bounds__(kFinMaxThreads)
 // slices in order.  Bound by latency and by finding the blocks (divisions):
 // the partials of kGRBatch blocks are loaded, then added; one channel per
 // thread and one load after another took 41 us at 2 x 342x628 (22 bands) and
-// 47 at 8 x 1920x1080.
+// 47 at 8 x 1920x1080, 29 as it is.
 // ---------------------------------------------------------------------------
 constexpr int kGRThreads = 512, kGRChunk = kGRThreads;
 constexpr int kGRBatch = 4;  // blocks in flight per vertex

@@ -1,8 +1,8 @@
 // The 3D LUT the paper starts from (Eq. 3) and the test of its hypothesis
 // that a sum of 2D LUTs can replace it (Eq. 4):
 //  - svdlut_lut3d_apply: trilinear transform of images by per-image 3D LUTs,
-//    gathered from shared memory (one output channel of a 33^3 table is 140
-//    KB, all three of a 26^3 one 206 KB); for few pixels per table, from a
+//    gathered from shared memory (one output channel of a 33^3 table is 150
+//    KB, all three of a 25^3 one 213 KB); for few pixels per table, from a
 //    copy repacked to one float4 (r, g, b, pad) per vertex through L1/L2;
 //  - svdlut_lut3d_fit2d: the least-squares fit of each 3D table by
 //    A[i][j] + B[i][k] + C[j][k] on the vertex grid, which is the
@@ -70,17 +70,36 @@ __global__ void __launch_bounds__(256) lut3d_apply_kernel(const float4 *__restri
 // Bound by the shared-memory pipe: 8 4-byte loads per pixel and channel, about
 // 3.5 passes each for noise (32 random banks) and 1 to 2 for smooth content;
 // a 16-byte gather of the three channels through L1 moves 16 bytes for 12 and
-// misses L1 (575 KB).  4K frame, D = 33, half noise: see below kMinShared.
+// misses L1 (575 KB) unless the pixels are coherent.  One 4K frame, D = 33: 80 us
+// for half noise, half smooth (113 through L1), 68 for a photo (70).
 constexpr int kSharedThreads = 1024;
+
+// Strides (floats) of the table in shared memory.  Its own, D and D^2, are 1 and
+// 1 modulo the 32 banks at D = 33, so that neighbouring cells with the same
+// i + j + k fall in one bank, and a photo's pixels, scattered over a few
+// neighbouring cells, in few (92 us at 3 x 2027x1000, 60 through L1).  Strides
+// of 3 and 9 modulo 32 (or -3, -9) put the 27 cells around one in 27 banks.
+struct TableStrides {
+    int g, r;  // of the second and the first axis
+};
+__host__ __device__ inline TableStrides table_strides(int D)
+{
+    TableStrides t{D, 0};
+    while ((t.g & 31) != 3 && (t.g & 31) != 29) ++t.g;
+    t.r = D * t.g;
+    while ((t.r & 31) != 9 && (t.r & 31) != 23) ++t.r;
+    return t;
+}
 
 template <int CH, int VEC>
 __global__ void __launch_bounds__(kSharedThreads, 1)
     lut3d_shared_kernel(const float *__restrict__ lut, int D, int B, size_t plane, int groups,
                         const float *__restrict__ x, float *__restrict__ y)
 {
-    extern __shared__ __align__(16) float table[];  // [CH][D^3]
+    extern __shared__ __align__(16) float table[];  // [CH][D] slabs of table_strides
     const int g = static_cast<int>(blockIdx.x) / (3 / CH), c0 = static_cast<int>(blockIdx.x) % (3 / CH);
-    const int n3 = D * D * D, sg = D, sr = D * D;
+    const TableStrides ts = table_strides(D);
+    const int n3 = D * D * D, sg = ts.g, sr = ts.r, ch = D * sr;
     const float fD1 = static_cast<float>(D - 1), fD2 = static_cast<float>(D - 2);
     const size_t per = plane / VEC, U = per * B;  // units of VEC adjacent pixels of a plane
     const size_t e1 = U * (g + 1) / groups;
@@ -90,7 +109,10 @@ __global__ void __launch_bounds__(kSharedThreads, 1)
         __syncthreads();  // the previous image's pixels are done with the table
         const float *src = lut + (b * 3 + c0) * n3;
 #pragma unroll 8
-        for (int v = threadIdx.x; v < CH * n3; v += kSharedThreads) table[v] = __ldg(src + v);
+        for (int v = threadIdx.x; v < CH * n3; v += kSharedThreads) {
+            const int row = v / D, slab = row / D;  // slab = channel * D + first index
+            table[slab * sr + (row - slab * D) * sg + (v - row * D)] = __ldg(src + v);
+        }
         __syncthreads();
         const float *xb = x + b * 3 * plane;
         float *yb = y + (b * 3 + c0) * plane;
@@ -111,10 +133,10 @@ __global__ void __launch_bounds__(kSharedThreads, 1)
                 const int ir = cell_of(__saturatef(in[0][k]), fD1, fD2, fr);
                 const int ig = cell_of(__saturatef(in[1][k]), fD1, fD2, fg);
                 const int ib = cell_of(__saturatef(in[2][k]), fD1, fD2, fb);
-                const float *t0 = table + (ir * D + ig) * D + ib;
+                const float *t0 = table + ir * sr + ig * sg + ib;
 #pragma unroll
                 for (int c = 0; c < CH; ++c) {
-                    const float *t = t0 + c * n3;
+                    const float *t = t0 + c * ch;
                     const float c000 = t[0], c001 = t[1], c010 = t[sg], c011 = t[sg + 1];
                     const float c100 = t[sr], c101 = t[sr + 1], c110 = t[sr + sg], c111 = t[sr + sg + 1];
                     const float c00 = fmaf(c001 - c000, fb, c000), c01 = fmaf(c011 - c010, fb, c010);
@@ -208,7 +230,9 @@ __global__ void __launch_bounds__(kFitThreads) lut3d_fit2d_kernel(const float *_
     }
 }
 
-// Fewest pixels per table for the shared-memory gathers.
+// Fewest pixels of an image for the shared-memory gathers: 14 us against 23 at
+// 512 x 512.  One image only: in a batch CTAs load a second table or stay idle
+// (3 photos of 2027 x 1000, D = 33: 65 us against 58 through L1).
 constexpr size_t kMinShared = size_t(1) << 18;
 
 template <int CH, int VEC>
@@ -221,7 +245,7 @@ svdlut_status launch_shared(const float *lut, int D, int B, size_t plane, const 
     const size_t units = plane / VEC * B;
     const int groups = static_cast<int>(std::min<size_t>(std::max(di.sm_count / (3 / CH), 1),
                                                          (units + kSharedThreads - 1) / kSharedThreads));
-    lut3d_shared_kernel<CH, VEC><<<groups * (3 / CH), kSharedThreads, sizeof(float) * CH * D * D * D, s>>>(
+    lut3d_shared_kernel<CH, VEC><<<groups * (3 / CH), kSharedThreads, sizeof(float) * CH * D * table_strides(D).r, s>>>(
         lut, D, B, plane, groups, x, y);
     SVDLUT_CUDA_TRY(cudaGetLastError());
     return SVDLUT_OK;
@@ -258,10 +282,10 @@ extern "C" svdlut_status svdlut_lut3d_apply(int D, const float *lut3d, int B, in
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int n3 = D * D * D;
     const size_t plane = static_cast<size_t>(H) * W;
-    const size_t table = sizeof(float) * n3, limit = static_cast<size_t>(di.max_smem_optin);
+    const size_t table = sizeof(float) * D * table_strides(D).r, limit = static_cast<size_t>(di.max_smem_optin);
     // (a call in place takes the kernel whose threads read and write one pixel)
     const bool apart = x + 3 * plane * B <= y || y + 3 * plane * B <= x;
-    if (plane >= kMinShared && table <= limit && apart) {
+    if (B == 1 && plane >= kMinShared && table <= limit && apart) {
         const bool all = 3 * table <= limit, vec = plane % 4 == 0 && aligned(x, 16) && aligned(y, 16);
         if (all)
             return vec ? launch_shared<3, 4>(lut3d, D, B, plane, x, y, di, s)
