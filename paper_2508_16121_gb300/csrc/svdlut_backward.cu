@@ -21,6 +21,7 @@
 #include <utility>
 #include <vector>
 #include <cmath>
+#include <cstdint>
 
 #include "apply_kernel.cuh"
 #include "apply_launch.cuh"
@@ -42,6 +43,7 @@ struct BwdArgs {
     float rW1, rH1;
     int strips;
     int vec;  // 16-byte loads allowed
+    int seg;  // LUT pass: lut_segment
 };
 
 // ---------------------------------------------------------------------------
@@ -74,7 +76,7 @@ struct BwdArgs {
 // warps update in turns: 660, 440 and 563 us, the hand-over's latency; 12
 // warps of this kernel: 580, 323, 460 us; the queue for every batch: 671,
 // 282, 491 us.
-// Output per part of CTA g and image b, in slot g + b (lut_slots): lut_part
+// Output per part of CTA g and image b, in slot lut_slot(g, b): lut_part
 // [slot][c][pair][D*D], sums_part[slot][c] (sum of dy_c).
 // ---------------------------------------------------------------------------
 constexpr int kLutGroups = 5, kLutWarps = 3 * kLutGroups;
@@ -93,14 +95,29 @@ __host__ __device__ inline size_t lut_grad_smem(int D)
 
 // Shares of the LUT pass: work units [share(g), share(g + 1)) belong to CTA g.
 __host__ __device__ inline long long lut_share(long long units, int G, int g) { return units * g / G; }
-// The slots of image b's parts, one per CTA that holds some of it: a CTA's next
-// image, and an image's next CTA, is the next slot.
-__host__ __device__ inline void lut_slots(long long per_image, int B, int G, int b, int &s0, int &s1)
+// The slot of CTA g's part of image b: a CTA's next image, and an image's next
+// CTA, is the next slot.  Where a share ends with an image, both are next at
+// once: with d = gcd(G, B) that is at every multiple of G / d shares (a segment)
+// = B / d images, so G shares of B images have at most G + B - d parts.
+__host__ __device__ inline int lut_segment(int G, int B)
+{
+    int a = G, b = B;
+    while (b) {
+        const int t = a % b;
+        a = b;
+        b = t;
+    }
+    return G / a;
+}
+__host__ __device__ inline int lut_slot(int g, int b, int seg) { return g + b - g / seg; }
+inline size_t lut_slot_count(int G, int B) { return static_cast<size_t>(G) + B - G / lut_segment(G, B); }
+// The slots of image b's parts, one per CTA that holds some of it.
+__host__ __device__ inline void lut_slots(long long per_image, int B, int G, int seg, int b, int &s0, int &s1)
 {
     const long long U = per_image * B;
     auto owner = [&](long long u) { return static_cast<int>(((u + 1) * G + U - 1) / U - 1); };
-    s0 = owner(per_image * b) + b;
-    s1 = owner(per_image * (b + 1) - 1) + b + 1;
+    s0 = lut_slot(owner(per_image * b), b, seg);
+    s1 = lut_slot(owner(per_image * (b + 1) - 1), b, seg) + 1;
 }
 
 // Adds the 12 sums of lanes with equal keys (key < 0: none) into the lowest
@@ -304,7 +321,7 @@ __global__ void __launch_bounds__(kLutThreads, 1)
         }
         __syncthreads();
         // CTA partial [c][pair][vertex]: sum the groups in order
-        const size_t slot = static_cast<size_t>(blockIdx.x) + b;
+        const size_t slot = lut_slot(static_cast<int>(blockIdx.x), b, a.seg);
         float *out = lut_part + slot * 9 * DD;
         for (int e = threadIdx.x; e < 9 * DD; e += kLutThreads) {
             const int c = e / (3 * DD), r = e - c * 3 * DD, q = r / DD, vtx = r - q * DD;
@@ -700,7 +717,7 @@ __device__ inline float block_sum(float v, float *red)
 struct FinArgs {
     const float *U, *S, *V, *lw;
     float *dU, *dS, *dV, *dlw;
-    int D, R, B, G;       // G: CTAs of the LUT pass
+    int D, R, B, G, seg;  // G: CTAs of the LUT pass; seg: lut_segment
     long long per_image;  // its work units per image
 };
 
@@ -715,7 +732,7 @@ __global__ void __launch_bounds__(kFinMaxThreads)
     const int cp = blockIdx.x, b = blockIdx.y, c = cp / 3, pair = cp - c * 3;
     const int D = f.D, R = f.R, DD = D * D, DR = D * R;
     int s0, s1;  // the image's slots
-    lut_slots(f.per_image, f.B, f.G, b, s0, s1);
+    lut_slots(f.per_image, f.B, f.G, f.seg, b, s0, s1);
     float *G = sm;  // [kFinParts][DD]: the parts' sums, then G = the gradient of the table in part 0
     float *U = sm + kFinParts * DD, *V = U + DR, *Q = V + DR, *S = Q + DR, *red = S + R;  // Q[i][r] = sum_j dT[i][j] V[j][r]
     const size_t t = static_cast<size_t>(b) * 9 + cp;
@@ -953,7 +970,7 @@ __global__ void __launch_bounds__(kGRThreads, 3)
 // dgrid_w[b][k] = (the slice partials of each plane summed in order, the sum
 // of dy_{k mod 3} over the image from the LUT pass partials: the bias).
 struct GridWsum {
-    int B, K, G, smax;
+    int B, K, G, seg, smax;
     int sl[3];
     float *dgw;
     long long per_image;
@@ -972,7 +989,7 @@ __global__ void grid_wsum_kernel(GridWsum f, const float *__restrict__ wpart, co
         for (int i = 0; i < f.sl[q]; ++i) s += p[i];
     } else {
         int s0, s1;
-        lut_slots(f.per_image, f.B, f.G, b, s0, s1);
+        lut_slots(f.per_image, f.B, f.G, f.seg, b, s0, s1);
 #pragma unroll 8
         for (int i = s0; i < s1; ++i) s += sums_part[static_cast<size_t>(i) * 3 + k % 3];
     }
@@ -1031,7 +1048,7 @@ static void layout_backward(const svdlut_dims *d, int B, BwdPlan *pl)
     const int D = d->D_t;
     size_t off = 0;
     pl->off_lut = off;
-    const size_t slots = static_cast<size_t>(B) + pl->G - 1;
+    const size_t slots = lut_slot_count(pl->G, B);
     off = align256(off + sizeof(float) * slots * 9 * D * D);
     pl->off_sums = off;
     off = align256(off + sizeof(float) * slots * 3);
@@ -1050,16 +1067,18 @@ static void layout_backward(const svdlut_dims *d, int B, BwdPlan *pl)
     pl->total = off;
 }
 
-// LUT pass: CTAs, at most max_g (one per SM); estimated time = rows a group
-// walks (its share of the batch's strips x rows, + a fixed cost of about 16 rows
-// per CTA: clearing the tables, writing the partial) + a row's time per 24
-// partials of an image that lut_finalize_kernel sums.
-static int plan_lut_ctas(int B, long long units, int max_g)
+// LUT pass: CTAs, at most max_g (one per SM) and with at most max_slots parts;
+// estimated time = rows a group walks (its share of the batch's strips x rows,
+// + a fixed cost of about 16 rows per CTA: clearing the tables, writing the
+// partial) + a row's time per 24 partials of an image that lut_finalize_kernel
+// sums.
+static int plan_lut_ctas(int B, long long units, int max_g, size_t max_slots)
 {
     const long long U = units * B;
     long long best_cost = -1;
     int best = 1;
     for (int G = 1; G <= std::min<long long>(U, max_g); ++G) {
+        if (lut_slot_count(G, B) > max_slots) continue;
         const long long cost = 24 * (((U + G - 1) / G + kLutGroups - 1) / kLutGroups + 16) + (G + B - 1) / B;
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
@@ -1072,11 +1091,11 @@ static int plan_lut_ctas(int B, long long units, int max_g)
 // Grid pass of a plan whose G is set: blocks of 128 x BH with as many row
 // groups as fit; bands minimise waves x (rows a warp walks + a fixed cost of
 // about 8 rows per block: clearing the tables, summing the warps, writing the
-// partial), ties go to the better-filled waves, and plans within
-// svdlut_backward_noalloc's scratch go before larger ones.  smallest: the
-// smallest workspace instead.  False if no block fits.
-static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit, bool smallest,
-                      BwdPlan *pl)
+// partial), ties go to the better-filled waves, and plans within ws_limit bytes
+// go before larger ones.  smallest: the smallest workspace instead.  False if
+// no block fits.
+static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit, size_t ws_limit,
+                      bool smallest, BwdPlan *pl)
 {
     const int Dsc = d->Dsc;
     const int strips = (W + kTileW - 1) / kTileW;
@@ -1107,7 +1126,7 @@ static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, s
         const double waves = std::ceil(static_cast<double>(T) / sm_count - 1e-9);
         const double fill = static_cast<double>(T) / (waves * sm_count);
         const double score = smallest ? -static_cast<double>(q.total)
-                                      : -waves * (gp.rpw + 8) + 1e-3 * fill - (q.total > kNoAllocScratchBytes ? 1e12 : 0.0);
+                                      : -waves * (gp.rpw + 8) + 1e-3 * fill - (q.total > ws_limit ? 1e12 : 0.0);
         if (!fits || score > best_score + 1e-12) {
             best_score = score;
             best = q;
@@ -1119,31 +1138,34 @@ static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, s
     return fits;
 }
 
+// ws_limit: bytes that the caller can give (svdlut_backward_noalloc's scratch;
+// SIZE_MAX for svdlut_backward, whose caller allocates what the plan wants).  A
+// plan beyond it gives way to one within it, if there is any: beside the smallest
+// grid plan the LUT CTAs whose parts there is room for, then the best grid plan
+// beside those.  CTAs that hold whole images, or images that are whole CTAs, want
+// the fewest parts: 154 images of 256 x 256 leave room for 154 parts, 77 CTAs of
+// two images each.
 static svdlut_status plan_backward(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit,
-                                   BwdPlan *pl)
+                                   size_t ws_limit, BwdPlan *pl)
 {
     pl->lut_smem = lut_grad_smem(d->D_t);
     if (pl->lut_smem > smem_limit) return fail(SVDLUT_ERR_UNSUPPORTED, "D_t=%d too large for the adjoint", d->D_t);
     pl->units = static_cast<long long>((W + kLutTileW - 1) / kLutTileW) * H;
-    pl->G = plan_lut_ctas(B, pl->units, sm_count);
-    if (!plan_grid(d, B, H, W, sm_count, smem_limit, false, pl))
+    pl->G = plan_lut_ctas(B, pl->units, sm_count, SIZE_MAX);
+    if (!plan_grid(d, B, H, W, sm_count, smem_limit, ws_limit, false, pl))
         return fail(SVDLUT_ERR_UNSUPPORTED, "grid vertices too dense for the adjoint's blocks");
-    if (pl->total > kNoAllocScratchBytes) {
-        // stay within svdlut_backward_noalloc's scratch where fewer LUT CTAs
-        // and the smallest grid plan do
+    if (pl->total > ws_limit) {
         BwdPlan q = *pl;
         q.G = 1;
-        plan_grid(d, B, H, W, sm_count, smem_limit, true, &q);
-        if (q.total <= kNoAllocScratchBytes) {
+        plan_grid(d, B, H, W, sm_count, smem_limit, ws_limit, true, &q);
+        if (q.total <= ws_limit) {
             const size_t per = sizeof(float) * (9 * static_cast<size_t>(d->D_t) * d->D_t + 3);
-            q.G = static_cast<int>(std::min<size_t>(pl->G, 1 + (kNoAllocScratchBytes - q.total) / per));
-            layout_backward(d, B, &q);
-            while (q.total > kNoAllocScratchBytes) {  // the parts' alignment
-                --q.G;
+            size_t slots = static_cast<size_t>(B) + (ws_limit - q.total) / per;
+            do {
+                q.G = plan_lut_ctas(B, q.units, sm_count, slots--);
                 layout_backward(d, B, &q);
-            }
-            q.G = plan_lut_ctas(B, q.units, q.G);
-            plan_grid(d, B, H, W, sm_count, smem_limit, false, &q);
+            } while (q.total > ws_limit);  // the parts' alignment
+            plan_grid(d, B, H, W, sm_count, smem_limit, ws_limit, false, &q);
             *pl = q;
         }
     }
@@ -1198,15 +1220,20 @@ static svdlut_status check_backward_args(const svdlut_dims *dims, const svdlut_p
 
 using namespace svdlut;
 
-extern "C" size_t svdlut_backward_workspace_size(const svdlut_dims *dims, int B, int H, int W)
+size_t svdlut::backward_workspace(const svdlut_dims *dims, int B, int H, int W, size_t ws_limit)
 {
     if (check_dims(dims) != SVDLUT_OK || B < 1 || H < 1 || W < 1) return 0;
     DeviceInfo di;
     if (device_info(&di) != SVDLUT_OK) return 0;
     BwdPlan pl;
-    if (plan_backward(dims, B, H, W, di.sm_count, static_cast<size_t>(di.max_smem_optin), &pl) != SVDLUT_OK)
+    if (plan_backward(dims, B, H, W, di.sm_count, static_cast<size_t>(di.max_smem_optin), ws_limit, &pl) != SVDLUT_OK)
         return 0;
     return pl.total;
+}
+
+extern "C" size_t svdlut_backward_workspace_size(const svdlut_dims *dims, int B, int H, int W)
+{
+    return backward_workspace(dims, B, H, W, SIZE_MAX);
 }
 
 extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_params *params, int B, int H,
@@ -1215,6 +1242,13 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
                                          svdlut_stream_t stream)
 {
     SVDLUT_TRACE("svdlut_backward");
+    return backward_limited(dims, params, B, H, W, x, dy, dx, grads, ws, ws_bytes, SIZE_MAX, stream);
+}
+
+svdlut_status svdlut::backward_limited(const svdlut_dims *dims, const svdlut_params *params, int B, int H, int W,
+                                       const float *x, const float *dy, float *dx, const svdlut_grads *grads,
+                                       void *ws, size_t ws_bytes, size_t ws_limit, svdlut_stream_t stream)
+{
     clear_error();
     svdlut_status st = check_backward_args(dims, params, B, H, W, x, dy);
     if (st != SVDLUT_OK) return st;
@@ -1237,7 +1271,7 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
     const bool want_lut = g.dU || g.dS || g.dV || g.dlut_w;
     const bool want_grid = dims->K > 0 && (g.dg_xy || g.dg_xc || g.dg_yc || g.dgrid_w);
     BwdPlan pl;
-    if ((st = plan_backward(dims, B, H, W, di.sm_count, smem_limit, &pl)) != SVDLUT_OK) return st;
+    if ((st = plan_backward(dims, B, H, W, di.sm_count, smem_limit, ws_limit, &pl)) != SVDLUT_OK) return st;
     const bool have_ws = ws && ws_bytes >= pl.total;
     if ((want_lut || want_grid) && !have_ws)
         return fail(SVDLUT_ERR_WORKSPACE, "workspace of %zu bytes needed (got %zu)", pl.total, ws ? ws_bytes : 0);
@@ -1273,6 +1307,7 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
     a.rH1 = H > 1 ? 1.0f / static_cast<float>(H - 1) : 0.f;
     a.strips = (W + kTileW - 1) / kTileW;
     a.vec = (W % 4 == 0) && aligned(x, 16) && aligned(dy, 16);
+    a.seg = lut_segment(pl.G, B);
 
     if ((st = allow_dynamic_smem(reinterpret_cast<const void *>(lut_grad_kernel), di.max_smem_optin, di.device)) !=
         SVDLUT_OK)
@@ -1291,7 +1326,7 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
         return st;
     if (want_lut) {
         FinArgs f{params->U, params->S, params->V, params->lut_w, g.dU, g.dS, g.dV, g.dlut_w,
-                  dims->D_t, dims->rank, B, pl.G, pl.units};
+                  dims->D_t, dims->rank, B, pl.G, a.seg, pl.units};
         const size_t fsm = sizeof(float) * fin_smem_floats(dims->D_t, dims->rank);
         if ((st = launch_pdl(lut_finalize_kernel, dim3(9, B), dim3(9 * B <= di.sm_count ? kFinMaxThreads : kFinMaxThreads / 2), fsm, s, f,
                              static_cast<const float *>(lut_part), static_cast<const float *>(sums_part))) != SVDLUT_OK)
@@ -1337,7 +1372,7 @@ extern "C" svdlut_status svdlut_backward(const svdlut_dims *dims, const svdlut_p
                              r, static_cast<const float *>(grid_part))) != SVDLUT_OK)
             return st;
         if (g.dgrid_w) {
-            GridWsum f{B, dims->K, pl.G, pl.smax, {pl.sl[0], pl.sl[1], pl.sl[2]}, g.dgrid_w, pl.units};
+            GridWsum f{B, dims->K, pl.G, a.seg, pl.smax, {pl.sl[0], pl.sl[1], pl.sl[2]}, g.dgrid_w, pl.units};
             const int n = B * dims->K * 4;
             if ((st = launch_pdl(grid_wsum_kernel, dim3((n + 255) / 256), dim3(256), 0, s, f,
                                  static_cast<const float *>(wpart), static_cast<const float *>(sums_part))) != SVDLUT_OK)

@@ -57,6 +57,14 @@ constexpr int kMaxDsc = 64;
 // Scratch space of svdlut_backward_noalloc (bytes).
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
 
+// svdlut_backward, and its workspace size, with a plan that stays within ws_limit
+// bytes of workspace where one does (SIZE_MAX: the fastest plan).  Both take the
+// same limit, so that they agree on the layout.
+size_t backward_workspace(const svdlut_dims *dims, int B, int H, int W, size_t ws_limit);
+svdlut_status backward_limited(const svdlut_dims *dims, const svdlut_params *params, int B, int H, int W,
+                               const float *x, const float *dy, float *dx, const svdlut_grads *grads, void *ws,
+                               size_t ws_bytes, size_t ws_limit, svdlut_stream_t stream);
+
 // Validate dims against the documented ranges.
 svdlut_status check_dims(const svdlut_dims *d);
 

@@ -96,7 +96,7 @@ extern "C" svdlut_status svdlut_backward_noalloc(const svdlut_dims *dims, const 
     void *ws = nullptr;
     size_t ws_bytes = 0;
     if (needs_ws) {
-        const size_t need = svdlut_backward_workspace_size(dims, B, H, W);
+        const size_t need = svdlut::backward_workspace(dims, B, H, W, kNoAllocScratchBytes);
         if (need == 0)  // bad arguments: let svdlut_backward report them
             return svdlut_backward(dims, params, B, H, W, x, dy, dx, grads, nullptr, 0, stream);
         if (need > kNoAllocScratchBytes)
@@ -110,5 +110,5 @@ extern "C" svdlut_status svdlut_backward_noalloc(const svdlut_dims *dims, const 
     }
     // Nothing in the scratch needs to start at zero: every pass writes the
     // parts it later reads.
-    return svdlut_backward(dims, params, B, H, W, x, dy, dx, grads, ws, ws_bytes, stream);
+    return svdlut::backward_limited(dims, params, B, H, W, x, dy, dx, grads, ws, ws_bytes, kNoAllocScratchBytes, stream);
 }
