@@ -1032,9 +1032,12 @@ static svdlut_status allow_dynamic_smem(const void *f, int max_optin, int device
     return SVDLUT_OK;
 }
 
-// Grid densities that the adjoint takes: 16 warps' xy, xc and yc vertices of a
-// block of BH rows within the shared memory (denser grids than about one
-// vertex per two pixels are refused).
+// Grid densities that the adjoint takes, a rule of the entry point and not what
+// the kernel could hold: 16 warps' xy, xc and yc vertices of a block of BH rows,
+// three channels each, in the shared memory (about one vertex per two pixels at
+// Dsc = 17).  Whatever it takes fits as a block of one row (plan_grid): one row
+// group's warps want 3 * (192 Dsc + nvyw (Dsc + nvx)) floats, and the rule bounds
+// 48 * nvyw (Dsc + nvx) by the shared memory.
 static bool grid_density_ok(int BH, int nvx, int H, int Dsy, int Dsc, size_t smem_limit)
 {
     const int nvyw = span_bound((BH + kWarps - 1) / kWarps, H, Dsy);
@@ -1092,35 +1095,36 @@ static int plan_lut_ctas(int B, long long units, int max_g, size_t max_slots)
 // groups as fit; bands minimise waves x (rows a warp walks + a fixed cost of
 // about 8 rows per block: clearing the tables, summing the warps, writing the
 // partial), ties go to the better-filled waves, and plans within ws_limit bytes
-// go before larger ones.  smallest: the smallest workspace instead.  False if
-// no block fits.
+// go before larger ones.  smallest: the smallest workspace instead.  Blocks have
+// at least about 16 rows; where the y vertices are so dense that no such block's
+// row groups hold theirs (Dsc = 64: six per image row), the tallest block that
+// fits.  False for densities that the adjoint does not take.
 static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, size_t smem_limit, size_t ws_limit,
                       bool smallest, BwdPlan *pl)
 {
     const int Dsc = d->Dsc;
-    const int strips = (W + kTileW - 1) / kTileW;
+    const int strips = (W + kTileW - 1) / kTileW, nvx = span_bound(kTileW, W, d->Dsx);
     const int max_bands = std::max(1, (H + kMinBlockH - 1) / kMinBlockH);
     BwdPlan best{};
-    bool fits = false;
+    bool taken = false, fits = false;
     double best_score = -1e30;
-    for (int bands = 1; bands <= max_bands; ++bands) {
+    auto consider = [&](int BH) {
         BwdPlan q = *pl;
         GridPlan &gp = q.gp;
-        gp.BH = (H + bands - 1) / bands;
-        gp.bands = (H + gp.BH - 1) / gp.BH;
-        gp.nvx = span_bound(kTileW, W, d->Dsx);
-        gp.nvy = span_bound(gp.BH, H, d->Dsy);
-        if (!grid_density_ok(gp.BH, gp.nvx, H, d->Dsy, Dsc, smem_limit)) continue;
+        gp.BH = BH;
+        gp.bands = (H + BH - 1) / BH;
+        gp.nvx = nvx;
+        gp.nvy = span_bound(BH, H, d->Dsy);
         for (gp.groups = kGridGroups; gp.groups > 0; --gp.groups) {
-            gp.rpw = (gp.BH + gp.groups - 1) / gp.groups;
+            gp.rpw = (BH + gp.groups - 1) / gp.groups;
             gp.nvyw = span_bound(gp.rpw, H, d->Dsy);
-            q.grid_smem = sizeof(float) * (static_cast<size_t>(grid_shared_floats(gp.nvx)) +
-                                           static_cast<size_t>(3 * gp.groups) * grid_warp_floats(gp.nvx, gp.nvyw, Dsc));
+            q.grid_smem = sizeof(float) * (static_cast<size_t>(grid_shared_floats(nvx)) +
+                                           static_cast<size_t>(3 * gp.groups) * grid_warp_floats(nvx, gp.nvyw, Dsc));
             if (q.grid_smem + 256 <= smem_limit) break;  // + the kernel's static row offsets
         }
-        if (gp.groups == 0) continue;
+        if (gp.groups == 0) return;
         gp.nblk = strips * gp.bands;
-        gp.blk_stride = grid_block_floats(gp.nvx, gp.nvy, Dsc);
+        gp.blk_stride = grid_block_floats(nvx, gp.nvy, Dsc);
         layout_backward(d, B, &q);
         const long long T = static_cast<long long>(B) * strips * gp.bands;
         const double waves = std::ceil(static_cast<double>(T) / sm_count - 1e-9);
@@ -1132,8 +1136,16 @@ static bool plan_grid(const svdlut_dims *d, int B, int H, int W, int sm_count, s
             best = q;
             fits = true;
         }
-        if (bands >= 4 * sm_count) break;
+    };
+    for (int bands = 1; bands <= max_bands; ++bands) {
+        const int BH = (H + bands - 1) / bands;
+        if (!grid_density_ok(BH, nvx, H, d->Dsy, Dsc, smem_limit)) continue;
+        taken = true;
+        consider(BH);
+        if (fits && bands >= 4 * sm_count) break;
     }
+    if (taken)
+        for (int BH = std::min(H, kMinBlockH); BH > 0 && !fits; --BH) consider(BH);
     if (fits) *pl = best;
     return fits;
 }

@@ -1,6 +1,7 @@
 """The adjoint's launch plans (no GPU needed): a program that includes the
 adjoint's source prints them for the sizes given, for a GPU of 152 SMs with 227
 KB of shared memory per CTA."""
+import math
 import subprocess
 
 import pytest
@@ -106,3 +107,36 @@ def test_every_part_has_its_slot(program):
              for per in (1, 5, 152, 1080) if G <= B * per]
     for c, (good,) in zip(cases, program("slots", cases)):
         assert good == 1, c
+
+
+def _span(extent, n, ds):
+    """Vertices that `extent` adjacent pixels of an axis of n touch, at most."""
+    if n <= 1:
+        return min(2, ds)
+    return min(ds, math.ceil((extent - 1) * ((ds - 1) / (n - 1))) + 3)
+
+
+def _taken(D, R, K, Dsx, Dsy, Dsc, B, H, W):
+    """The densities that the adjoint takes: in some block of a band of the
+    image, 16 warps' vertices of three channels within the shared memory."""
+    nvx = _span(128, W, Dsx)
+    for bands in range(1, max(1, -(-H // 16)) + 1):
+        BH = -(-H // bands)
+        ny = _span(-(-BH // 16), H, Dsy)
+        if 4 * 16 * ((3 * (ny * nvx + (nvx + ny) * Dsc) + 3) // 4 * 4) + 256 <= 227 * 1024:
+            return True
+    return False
+
+
+def test_dense_grids_are_taken(program):
+    """Many y vertices per image row, up to the densest grids that the adjoint
+    takes: every one of those has a plan whose blocks fit."""
+    cases = [(17, 8, 6, 17, 129, 64, 1, 16, 256)]
+    for Dsc in (2, 5, 9, 17, 24, 33, 48, 64):
+        for H, W in ((1, 1), (3, 70), (16, 256), (20, 130), (37, 300), (200, 90)):
+            for per_row in (1, 3, 6, 8, 12, 16, 24, 32, 48, 64):
+                for Dsx in (2, 5, max(2, W // 8), max(2, W // 2)):
+                    cases.append((9, 3, 4, Dsx, max(2, H * per_row), Dsc, 2, H, W))
+    assert any(_taken(*c) for c in cases) and not all(_taken(*c) for c in cases)
+    for c, p in zip(cases, program("plan", cases)):
+        assert (p[0] == 0) == _taken(*c), (c, p)
