@@ -698,7 +698,9 @@ __global__ void __launch_bounds__(kGridThreads, 1)
 // summed in up to kFinParts contiguous parts, side by side, kFinBatch loads at a
 // time, then the parts in order: two images' 152 partials on 18 CTAs were bound
 // by the latency of one chain of loads per vertex (76 us at 2 x 342x628; 17 us at
-// 8 x 1920x1080 and at 64 x 256x256 as it is, 27 and 20 before).
+// 8 x 1920x1080 and at 64 x 256x256 as it is, 27 and 20 before).  Two CTAs of 1024
+// threads per SM, thus 32 registers: 45 leave two CTAs of 512 instead of four, and
+// svdlut_backward at 64 x 256x256 takes 340 us instead of 337.
 // ---------------------------------------------------------------------------
 constexpr int kFinMaxThreads = 1024, kFinParts = 8, kFinBatch = 8;
 
@@ -723,7 +725,7 @@ struct FinArgs {
 
 __host__ __device__ inline int fin_smem_floats(int D, int R) { return kFinParts * D * D + 3 * D * R + R + kFinMaxThreads / 32; }
 
-__global__ void __launch_bounds__(kFinMaxThreads)
+__global__ void __launch_bounds__(kFinMaxThreads, 2)
     lut_finalize_kernel(FinArgs f, const float *__restrict__ lut_part, const float *__restrict__ sums_part)
 {
     pdl_enter();
