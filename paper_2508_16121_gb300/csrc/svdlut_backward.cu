@@ -698,9 +698,10 @@ __global__ void __launch_bounds__(kGridThreads, 1)
 // summed in up to kFinParts contiguous parts, side by side, kFinBatch loads at a
 // time, then the parts in order: two images' 152 partials on 18 CTAs were bound
 // by the latency of one chain of loads per vertex (76 us at 2 x 342x628; 17 us at
-// 8 x 1920x1080 and at 64 x 256x256 as it is, 27 and 20 before).  Two CTAs of 1024
-// threads per SM, thus 32 registers: 45 leave two CTAs of 512 instead of four, and
-// svdlut_backward at 64 x 256x256 takes 340 us instead of 337.
+// 8 x 1920x1080 and at 64 x 256x256 as it is, 27 and 20 before).  One thread
+// works out the image's slots: with that in every thread the kernel took 45
+// registers instead of 32, two CTAs of 512 threads per SM instead of four, and
+// svdlut_backward at 64 x 256x256 340 us instead of 337.
 // ---------------------------------------------------------------------------
 constexpr int kFinMaxThreads = 1024, kFinParts = 8, kFinBatch = 8;
 
@@ -725,7 +726,7 @@ struct FinArgs {
 
 __host__ __device__ inline int fin_smem_floats(int D, int R) { return kFinParts * D * D + 3 * D * R + R + kFinMaxThreads / 32; }
 
-__global__ void __launch_bounds__(kFinMaxThreads, 2)
+__global__ void __launch_bounds__(kFinMaxThreads)
     lut_finalize_kernel(FinArgs f, const float *__restrict__ lut_part, const float *__restrict__ sums_part)
 {
     pdl_enter();
@@ -733,8 +734,10 @@ __global__ void __launch_bounds__(kFinMaxThreads, 2)
     const int nthr = blockDim.x;
     const int cp = blockIdx.x, b = blockIdx.y, c = cp / 3, pair = cp - c * 3;
     const int D = f.D, R = f.R, DD = D * D, DR = D * R;
-    int s0, s1;  // the image's slots
-    lut_slots(f.per_image, f.B, f.G, f.seg, b, s0, s1);
+    __shared__ int slots[2];  // the image's
+    if (threadIdx.x == 0) lut_slots(f.per_image, f.B, f.G, f.seg, b, slots[0], slots[1]);
+    __syncthreads();
+    const int s0 = slots[0], s1 = slots[1];
     float *G = sm;  // [kFinParts][DD]: the parts' sums, then G = the gradient of the table in part 0
     float *U = sm + kFinParts * DD, *V = U + DR, *Q = V + DR, *S = Q + DR, *red = S + R;  // Q[i][r] = sum_j dT[i][j] V[j][r]
     const size_t t = static_cast<size_t>(b) * 9 + cp;
