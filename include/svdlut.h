@@ -172,11 +172,13 @@ svdlut_status svdlut_apply_cfg(const svdlut_dims *dims, const svdlut_params *par
  * coefficient form of the bilinear interpolation (Supp. Eq. 15), folds the
  * grid slices per output channel (Supp. Eqs. 21-22) and sums the biases; the
  * transform kernel, launched as its programmatic dependent, copies its part
- * of those tables into shared memory.  The result is bit-identical to
- * svdlut_apply.
+ * of those tables into shared memory.  A launch of 16 images or more whose CTAs
+ * can build the LUTs as quickly themselves (rank 8, 16-byte aligned factors)
+ * takes the folded grids alone from the workspace, or, up to 2^19 pixels in all,
+ * nothing.  The result is bit-identical to svdlut_apply.
  * ws: device memory of at least svdlut_apply_workspace_size(dims, B) bytes,
  * 256-byte aligned, not overlapping x or y; its contents on entry do not
- * matter and are overwritten; concurrent calls must use different workspaces.
+ * matter and may be overwritten; concurrent calls must use different workspaces.
  * cfg may be NULL.
  * Errors: those of svdlut_apply_cfg; WORKSPACE (NULL or too small);
  * INVALID_ARG (misaligned or overlapping workspace).
@@ -197,7 +199,7 @@ size_t svdlut_apply_workspace_size(const svdlut_dims *dims, int B);
  * launch per 64 images.  imgs is a HOST array of n descriptors (read during the
  * call only).  With the queue schedule the images' blocks are taken from a
  * counter in ws; either way the call is capturable in a CUDA graph (a 4-byte
- * memset, for the queue, + one kernel per 64 images).
+ * memset, for the queue, + one kernel, or two with the tables, per 64 images).
  * ws: device memory of svdlut_batched_workspace_size(n) bytes, 4-byte aligned;
  * concurrent calls must use different workspaces.  cfg may be NULL.
  * Errors: INVALID_ARG (a bad image, reported with its index), WORKSPACE,
@@ -216,7 +218,8 @@ size_t svdlut_batched_workspace_size(int n);
  * cell tables and folded grids of svdlut_apply_ws, computed once per call by
  * one small kernel and copied into each CTA); 0 on bad arguments.  A
  * workspace of at least this size, 256-byte aligned, makes
- * svdlut_apply_batched use them (same results, bit for bit). */
+ * svdlut_apply_batched use them where svdlut_apply_ws would (same results, bit
+ * for bit). */
 size_t svdlut_batched_tables_workspace_size(const svdlut_image *imgs, int n);
 
 /*

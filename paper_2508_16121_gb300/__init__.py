@@ -110,6 +110,27 @@ def _stream_ptr(stream=None):
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
+# Calls that this binding's own work bounds: one launch without a workspace takes
+# 18 to 20 us of host time, two with one from the allocator 24 to 27, while the GPU
+# needs 10 to 20 (2 or 3 of them more without the tables).  us per call, with and
+# without: 64 x 64 23.7 / 19.8, 724 x 724 23.9 / 20.3, 15 x 180x190 25.7 / 21.8;
+# but 853 x 1279 24.9 / 26.1, and at rank 16 15 x 180x190 28.6 / 31.3.  A replayed
+# graph has no host time: a call that is captured takes the tables.
+_CALL_BOUND_PX = 1 << 19
+_CALL_BOUND_IMAGES = 15
+_CALL_BOUND_RANK = 8
+
+
+def _call_bound(B, H, W, d, stream):
+    if B > _CALL_BOUND_IMAGES or B * H * W > _CALL_BOUND_PX or d.rank > _CALL_BOUND_RANK:
+        return False
+    torch = _torch()
+    if stream is None:
+        return not torch.cuda.is_current_stream_capturing()
+    with torch.cuda.stream(stream):
+        return not torch.cuda.is_current_stream_capturing()
+
+
 def apply(x, params, out=None, stream=None, ctas=None, workspace=True):
     """Fused SVDLUT apply (Eq. 10).  x: CUDA tensor [B,3,H,W] or [3,H,W],
     float32 or uint8, contiguous.  params: dict of float32 CUDA tensors with
@@ -117,9 +138,10 @@ def apply(x, params, out=None, stream=None, ctas=None, workspace=True):
     x's shape and dtype.  ctas: persistent CTAs to use (default one per SM).
     workspace: True (default) runs svdlut_apply_ws, whose per-image tables
     are precomputed once into a workspace taken from PyTorch's allocator on
-    the call's stream; a uint8 CUDA tensor of svdlut_apply_workspace_size
-    bytes is used as given; False runs svdlut_apply / svdlut_apply_cfg
-    (every CTA rebuilds the tables itself)."""
+    the call's stream (or, where that is quicker, as False: _call_bound); a
+    uint8 CUDA tensor of svdlut_apply_workspace_size bytes is used as given;
+    False runs svdlut_apply / svdlut_apply_cfg (every CTA rebuilds the tables
+    itself).  The results are the same bits."""
     torch = _torch()
     squeeze = x.dim() == 3
     xb = x.unsqueeze(0) if squeeze else x
@@ -139,6 +161,8 @@ def apply(x, params, out=None, stream=None, ctas=None, workspace=True):
     if out is not None and (y.shape != xb.shape or y.dtype != xb.dtype or not y.is_contiguous()):
         raise ValueError("out must match x in shape and dtype")
     lib = _lib.load()
+    if workspace is True and _call_bound(B, H, W, d, stream):
+        workspace = False
     if workspace is not False:
         if sizes.table_bytes is None:
             sizes.table_bytes = lib.svdlut_apply_workspace_size(d, 1)

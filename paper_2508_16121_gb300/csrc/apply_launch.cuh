@@ -184,27 +184,30 @@ bool factors_in_ctas(const LaunchArgs<N> &a)
     return true;
 }
 
-// Launches prep_kernel for planned args where it pays and sets a.pre.  Device
-// times of one launch with everything built in the CTAs / everything from
-// prep_kernel / the folded grids from prep_kernel, us:
-//   1 x 64x64     12.7 / 10.1 / 12.1    16 x 256x256  27.7 / 28.0 / 28.3
-//   1 x 853x1279  27.6 / 26.1 / 27.3    30 x 256x256  45.9 / 47.9 / 46.3
-//   1 x 4K        99.4 / 94.9 / 98.0    64 x 256x256  84.4 / 90.2 / 84.5
-//   4 x 1080p u8  99.1 / 97.2 / 98.4    77 x 190x558 u8  249 / 262 / 238
-// Few images: all CTAs copy one table while a few build it.  From kManyImages
-// on the tables cost as much as they save, the folds still pay.  Up to
-// kLaunchBoundPx pixels the call is bound by its launches (20 us of host time
-// with one, 23 with two), so it makes one.
+// Launches prep_kernel for planned args where it pays on the GPU and sets a.pre.
+// Device times of a call in a CUDA graph with everything built in the CTAs /
+// everything from prep_kernel / the folded grids from prep_kernel, float images,
+// us:
+//   1 x 64x64     12.5 /  9.9 / 12.2    16 x 64x64    15.2 / 14.6 / 13.9
+//   1 x 512x512   14.1 / 12.4 / 14.6    16 x 128x128  15.7 / 16.3 / 17.0
+//   1 x 853x1279  25.3 / 23.3 / 26.4    16 x 256x256  27.6 / 28.1 / 29.0
+//   1 x 4K        99.4 / 94.3 / 97.6    32 x 64x64    18.3 / 20.2 / 19.3
+//   8 x 64x64     13.6 / 10.5 / 13.0    64 x 90x90    33.4 / 39.9 / 34.9
+//   15 x 64x64    14.8 / 13.8 / 13.8    64 x 256x256  87.7 / 97.4 / 88.5
+//   15 x 128x128  15.4 / 15.8 / 16.1    77 x 190x558 (8-bit) 249 / 262 / 238
+// Few images: all CTAs copy one table while a few build it.  From kManyImages on
+// the tables cost as much as they save; the folds pay where the images are large
+// (from kFoldPx pixels of a launch: no more than 1 % lost, up to 5 % won).
 constexpr int kManyImages = 16;
-constexpr double kLaunchBoundPx = 512.0 * 1024.0;
+constexpr double kFoldPx = 512.0 * 1024.0;
 template <int N>
 svdlut_status launch_tables(LaunchArgs<N> &a, int sm_count, cudaStream_t s)
 {
     double px = 0;
     for (int i = 0; i < a.n; ++i) px += static_cast<double>(a.img[i].H) * a.img[i].W;
-    const bool in_ctas = factors_in_ctas(a);
-    if (in_ctas && px <= kLaunchBoundPx) return SVDLUT_OK;
-    a.pre = in_ctas && a.n >= kManyImages && all_fast_rows(a) ? kPreFolds : kPreAll;
+    const bool in_ctas = a.n >= kManyImages && factors_in_ctas(a);
+    if (in_ctas && px <= kFoldPx) return SVDLUT_OK;
+    a.pre = in_ctas && all_fast_rows(a) ? kPreFolds : kPreAll;
     return launch_prep(a, sm_count, s, a.pre == kPreAll);
 }
 
