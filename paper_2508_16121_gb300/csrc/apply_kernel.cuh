@@ -521,8 +521,16 @@ __host__ __device__ inline int prologue_floats_n(int D, int R, int pairs)
 
 // 16- and 4-byte asynchronous global -> shared copies (cp.async; L2 only for
 // 16 bytes) and the wait for all of this thread's copies.
-__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+__device__ __forceinline__ void cp_async16(unsigned int *check, void *dst, const void *src)
 {
+#ifdef SVDLUT_CHECK_BOUNDS
+    if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) != 0) {
+        check_record(check, kChkAlign, static_cast<unsigned int>(reinterpret_cast<uintptr_t>(src)), 16u);
+        return;
+    }
+#else
+    (void)check;
+#endif
     const unsigned int s = static_cast<unsigned int>(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(src) : "memory");
 }
@@ -572,15 +580,8 @@ __device__ inline void build_luts(const ImgDesc &d, float4 *lcell, float *tmp, f
                 const int cp = c * 3 + pp;
                 float *du = sU + slot * DRp + i * Rp + 4 * q, *dv = sV + slot * DRp + i * Rp + 4 * q;
                 const float *su = d.U + cp * DR + i * R + 4 * q, *sv = d.V + cp * DR + i * R + 4 * q;
-#ifdef SVDLUT_CHECK_BOUNDS
-                if (((reinterpret_cast<uintptr_t>(du) | reinterpret_cast<uintptr_t>(dv) |
-                      reinterpret_cast<uintptr_t>(su) | reinterpret_cast<uintptr_t>(sv)) & 15) != 0) {
-                    check_record(check, kChkAlign, static_cast<unsigned int>(reinterpret_cast<uintptr_t>(su)), 16u);
-                    continue;
-                }
-#endif
-                cp_async16(du, su);
-                cp_async16(dv, sv);
+                cp_async16(check, du, su);
+                cp_async16(check, dv, sv);
             }
             for (int e = tid; e < nf * (R + 1); e += kThreads) {
                 const int slot = e / (R + 1), r = e - slot * (R + 1);
@@ -687,16 +688,16 @@ __host__ __device__ __forceinline__ bool fast_factors_ok(const ImgDesc &d)
 
 // Issues the copies of image d's factors to buf: U, V [9][D][kFastRp], S
 // [9][8], lut_w [3][4]; and the summed biases.
-__device__ inline void copy_factors(const ImgDesc &d, float *buf, float *misc)
+__device__ inline void copy_factors(const ImgDesc &d, float *buf, float *misc, unsigned int *check)
 {
     const int tid = threadIdx.x, nrow = 9 * d.D, half = nrow * kFastRp;
     for (int e = tid; e < nrow * 2; e += kThreads) {  // 16-byte chunks of the rows
         const int row = e >> 1, q = 4 * (e & 1);
-        cp_async16(buf + row * kFastRp + q, d.U + row * kFastRank + q);
-        cp_async16(buf + half + row * kFastRp + q, d.V + row * kFastRank + q);
+        cp_async16(check, buf + row * kFastRp + q, d.U + row * kFastRank + q);
+        cp_async16(check, buf + half + row * kFastRp + q, d.V + row * kFastRank + q);
     }
-    if (tid < 18) cp_async16(buf + 2 * half + 4 * tid, d.S + 4 * tid);
-    else if (tid < 21) cp_async16(buf + 2 * half + 4 * tid, d.lw + 4 * (tid - 18));
+    if (tid < 18) cp_async16(check, buf + 2 * half + 4 * tid, d.S + 4 * tid);
+    else if (tid < 21) cp_async16(check, buf + 2 * half + 4 * tid, d.lw + 4 * (tid - 18));
     else if (tid >= 32 && tid < 35) {
         const int c = tid - 32;
         float b = __ldg(d.lw + c * 4 + 3);
@@ -975,7 +976,7 @@ __device__ __forceinline__ int quot(int n, float rm) { return static_cast<int>((
 // folded slices of its footprint (4-byte asynchronous copies).  The caller
 // waits for the copies.
 __device__ inline void setup_pre(const ImgDesc &d, const BlockGeom &g, const BlockBufs &b, float4 *lcell,
-                                 float *misc, bool rebuild)
+                                 float *misc, bool rebuild, unsigned int *check)
 {
     const int tid = threadIdx.x;
     const int nvx = g.nvx, nvy = g.nvy, Dsc = d.Dsc, Dsx = d.Dsx, Dsy = d.Dsy;
@@ -990,7 +991,7 @@ __device__ inline void setup_pre(const ImgDesc &d, const BlockGeom &g, const Blo
         const int rot = static_cast<int>((static_cast<long long>(n4) * blockIdx.x) / gridDim.x);
         for (int e = tid; e < n4; e += kThreads) {
             const int f = e + rot < n4 ? e + rot : e + rot - n4;
-            cp_async16(lcell + f, src + f);
+            cp_async16(check, lcell + f, src + f);
         }
         if (tid < 3) misc[kMaxK * 4 + tid] = __ldg(d.pfold + pfold_floats(Dsx, Dsy, Dsc) + tid);
     }
@@ -1425,7 +1426,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                 asm volatile("griddepcontrol.wait;\n" ::: "memory");
                 pre_wait = false;
             }
-            setup_pre(d, g, b, lcell, misc, im != cur_im);
+            setup_pre(d, g, b, lcell, misc, im != cur_im, a.check);
             cp_async_wait_all();
             __syncthreads();
         }
@@ -1433,7 +1434,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
             // pixels and factors are inputs of the call, complete before the
             // launch; the folded grids come after the wait for prep_kernel
             if (im != cur_im) {
-                copy_factors(d, b.xcol, misc);
+                copy_factors(d, b.xcol, misc, a.check);
                 cp_async_wait_all();
                 __syncthreads();
                 build_cells(d.D, b.xcol, lcell);
@@ -1443,7 +1444,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                 asm volatile("griddepcontrol.wait;\n" ::: "memory");
                 pre_wait = false;
             }
-            setup_pre(d, g, b, lcell, misc, false);
+            setup_pre(d, g, b, lcell, misc, false, a.check);
             cp_async_wait_all();
             __syncthreads();
         }
@@ -1452,7 +1453,7 @@ __global__ void __launch_bounds__(kThreads, 1) apply_kernel(const __grid_constan
                              (b.xcol - scratch) + fast_factor_floats(d.D) <= a.scratch_floats;
         if constexpr (PRE == kPreNone) {
             if (overlap) {
-                copy_factors(d, b.xcol, misc);
+                copy_factors(d, b.xcol, misc, a.check);
             } else if (im != cur_im) {
                 build_luts(d, lcell, scratch, misc, a.scratch_floats, a.check);
                 __syncthreads();
