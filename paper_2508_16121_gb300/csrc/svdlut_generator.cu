@@ -1868,13 +1868,16 @@ extern "C" svdlut_status svdlut_mse(const float *y, const float *target, size_t 
     clear_error();
     if (!y || !target || !loss || n == 0) return fail(SVDLUT_ERR_INVALID_ARG, "mse: null buffer or n = 0");
     const bool vec = aligned(y, 16) && aligned(target, 16) && (!dy || aligned(dy, 16));
-    const int nb = std::min(blocks_for(vec ? (n + 3) / 4 : n), 152 * kMseCtas);
-    const size_t need = sizeof(float) * static_cast<size_t>(std::min(blocks_for(n), 1024));  // at least nb
+    const size_t need = sizeof(float) * static_cast<size_t>(std::min(blocks_for(n), 1024));
     if (!ws || ws_bytes < need) return fail(SVDLUT_ERR_WORKSPACE, "mse: workspace of %zu bytes needed", need);
+    DeviceInfo di;
+    svdlut_status st = device_info(&di);
+    if (st != SVDLUT_OK) return st;
+    const int nb = std::min(blocks_for(vec ? (n + 3) / 4 : n), std::min(di.sm_count * kMseCtas, 1024));  // need at most
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     float *part = static_cast<float *>(ws);
-    const svdlut_status st = vec ? launch_pdl(mse_kernel<4>, dim3(nb), dim3(256), 0, s, y, target, n, dy, part)
-                                 : launch_pdl(mse_kernel<1>, dim3(nb), dim3(256), 0, s, y, target, n, dy, part);
+    st = vec ? launch_pdl(mse_kernel<4>, dim3(nb), dim3(256), 0, s, y, target, n, dy, part)
+             : launch_pdl(mse_kernel<1>, dim3(nb), dim3(256), 0, s, y, target, n, dy, part);
     if (st != SVDLUT_OK) return st;
     return launch_pdl(mse_final_kernel, dim3(1), dim3(32), 0, s, static_cast<const float *>(part), nb, n, loss);
 }
