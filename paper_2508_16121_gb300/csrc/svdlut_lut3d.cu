@@ -1,9 +1,10 @@
 // The 3D LUT the paper starts from (Eq. 3) and the test of its hypothesis
 // that a sum of 2D LUTs can replace it (Eq. 4):
-//  - svdlut_lut3d_apply: trilinear transform of images by per-image 3D LUTs,
-//    gathered from shared memory (one output channel of a 33^3 table is 150
-//    KB, all three of a 25^3 one 213 KB); for few pixels per table, from a
-//    copy repacked to one float4 (r, g, b, pad) per vertex through L1/L2;
+//  - svdlut_lut3d_apply: trilinear transform of images by per-image 3D LUTs;
+//    one large image's gathers come from shared memory (one output channel of
+//    a 33^3 table is 150 KB, all three of a 25^3 one 213 KB), those of small
+//    images and of batches from a copy repacked to one float4 (r, g, b, pad)
+//    per vertex, through L1/L2;
 //  - svdlut_lut3d_fit2d: the least-squares fit of each 3D table by
 //    A[i][j] + B[i][k] + C[j][k] on the vertex grid, which is the
 //    second-order ANOVA projection fit = m_ij. + m_i.k + m_.jk - m_i.. -
@@ -63,15 +64,15 @@ __global__ void __launch_bounds__(256) lut3d_apply_kernel(const float4 *__restri
     }
 }
 
-// Gathers from shared memory.  CH channels of the table per CTA: all three
-// where they fit, else one, and every third CTA then walks the same pixels (two
-// of the three read them from L2).  Group g of G takes the g-th share of the
-// batch's pixels, one image's part after another, and loads that image's table.
-// Bound by the shared-memory pipe: 8 4-byte loads per pixel and channel, about
-// 3.5 passes each for noise (32 random banks) and 1 to 2 for smooth content;
-// a 16-byte gather of the three channels through L1 moves 16 bytes for 12 and
-// misses L1 (575 KB) unless the pixels are coherent.  One 4K frame, D = 33: 80 us
-// for half noise, half smooth (113 through L1), 68 for a photo (70).
+// Gathers from shared memory, for one image.  CH channels of the table per CTA:
+// all three where they fit, else one, and every third CTA then walks the same
+// pixels (two of the three read them from L2).  Group g of the groups takes the
+// g-th share of the pixels.  Bound by the shared-memory pipe: 8 4-byte loads per
+// pixel and channel, about 3.5 passes each for noise (32 random banks) and 1 to 2
+// for smooth content; a 16-byte gather of the three channels through L1 moves 16
+// bytes for 12 and misses L1 (575 KB) unless the pixels are coherent.  One 4K
+// frame, D = 33: 81 us for half noise, half smooth (113 through L1), 71 for a
+// photo (70).
 constexpr int kSharedThreads = 1024;
 
 // Strides (floats) of the table in shared memory.  Its own, D and D^2, are 1 and
@@ -93,66 +94,59 @@ __host__ __device__ inline TableStrides table_strides(int D)
 
 template <int CH, int VEC>
 __global__ void __launch_bounds__(kSharedThreads, 1)
-    lut3d_shared_kernel(const float *__restrict__ lut, int D, int B, size_t plane, int groups,
-                        const float *__restrict__ x, float *__restrict__ y)
+    lut3d_shared_kernel(const float *__restrict__ lut, int D, size_t plane, int groups, const float *__restrict__ x,
+                        float *__restrict__ y)
 {
     extern __shared__ __align__(16) float table[];  // [CH][D] slabs of table_strides
     const int g = static_cast<int>(blockIdx.x) / (3 / CH), c0 = static_cast<int>(blockIdx.x) % (3 / CH);
     const TableStrides ts = table_strides(D);
     const int n3 = D * D * D, sg = ts.g, sr = ts.r, ch = D * sr;
     const float fD1 = static_cast<float>(D - 1), fD2 = static_cast<float>(D - 2);
-    const size_t per = plane / VEC, U = per * B;  // units of VEC adjacent pixels of a plane
-    const size_t e1 = U * (g + 1) / groups;
-    for (size_t e0 = U * g / groups; e0 < e1;) {
-        const size_t b = e0 / per, p0 = e0 - b * per, p1 = min(e1 - b * per, per);
-        e0 = b * per + p1;
-        __syncthreads();  // the previous image's pixels are done with the table
-        const float *src = lut + (b * 3 + c0) * n3;
+    const float *src = lut + c0 * n3;
 #pragma unroll 8
-        for (int v = threadIdx.x; v < CH * n3; v += kSharedThreads) {
-            const int row = v / D, slab = row / D;  // slab = channel * D + first index
-            table[slab * sr + (row - slab * D) * sg + (v - row * D)] = __ldg(src + v);
+    for (int v = threadIdx.x; v < CH * n3; v += kSharedThreads) {
+        const int row = v / D, slab = row / D;  // slab = channel * D + first index
+        table[slab * sr + (row - slab * D) * sg + (v - row * D)] = __ldg(src + v);
+    }
+    __syncthreads();
+    y += c0 * plane;
+    const size_t units = plane / VEC, p1 = units * (g + 1) / groups;  // units of VEC adjacent pixels of a plane
+    for (size_t p = units * g / groups + threadIdx.x; p < p1; p += kSharedThreads) {
+        float in[3][VEC], out[CH][VEC];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if constexpr (VEC == 4) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(x + c * plane) + p);
+                in[c][0] = v.x, in[c][1] = v.y, in[c][2] = v.z, in[c][3] = v.w;
+            } else {
+                in[c][0] = __ldg(x + c * plane + p);
+            }
         }
-        __syncthreads();
-        const float *xb = x + b * 3 * plane;
-        float *yb = y + (b * 3 + c0) * plane;
-        for (size_t p = p0 + threadIdx.x; p < p1; p += kSharedThreads) {
-            float in[3][VEC], out[CH][VEC];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                if constexpr (VEC == 4) {
-                    const float4 v = __ldg(reinterpret_cast<const float4 *>(xb + c * plane) + p);
-                    in[c][0] = v.x, in[c][1] = v.y, in[c][2] = v.z, in[c][3] = v.w;
-                } else {
-                    in[c][0] = __ldg(xb + c * plane + p);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < VEC; ++k) {
-                float fr, fg, fb;
-                const int ir = cell_of(__saturatef(in[0][k]), fD1, fD2, fr);
-                const int ig = cell_of(__saturatef(in[1][k]), fD1, fD2, fg);
-                const int ib = cell_of(__saturatef(in[2][k]), fD1, fD2, fb);
-                const float *t0 = table + ir * sr + ig * sg + ib;
-#pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    const float *t = t0 + c * ch;
-                    const float c000 = t[0], c001 = t[1], c010 = t[sg], c011 = t[sg + 1];
-                    const float c100 = t[sr], c101 = t[sr + 1], c110 = t[sr + sg], c111 = t[sr + sg + 1];
-                    const float c00 = fmaf(c001 - c000, fb, c000), c01 = fmaf(c011 - c010, fb, c010);
-                    const float c10 = fmaf(c101 - c100, fb, c100), c11 = fmaf(c111 - c110, fb, c110);
-                    const float lo = fmaf(c01 - c00, fg, c00), hi = fmaf(c11 - c10, fg, c10);
-                    out[c][k] = fmaf(hi - lo, fr, lo);
-                }
-            }
+        for (int k = 0; k < VEC; ++k) {
+            float fr, fg, fb;
+            const int ir = cell_of(__saturatef(in[0][k]), fD1, fD2, fr);
+            const int ig = cell_of(__saturatef(in[1][k]), fD1, fD2, fg);
+            const int ib = cell_of(__saturatef(in[2][k]), fD1, fD2, fb);
+            const float *t0 = table + ir * sr + ig * sg + ib;
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
-                if constexpr (VEC == 4)
-                    __stcs(reinterpret_cast<float4 *>(yb + c * plane) + p,
-                           make_float4(out[c][0], out[c][1], out[c][2], out[c][3]));
-                else
-                    __stcs(yb + c * plane + p, out[c][0]);
+                const float *t = t0 + c * ch;
+                const float c000 = t[0], c001 = t[1], c010 = t[sg], c011 = t[sg + 1];
+                const float c100 = t[sr], c101 = t[sr + 1], c110 = t[sr + sg], c111 = t[sr + sg + 1];
+                const float c00 = fmaf(c001 - c000, fb, c000), c01 = fmaf(c011 - c010, fb, c010);
+                const float c10 = fmaf(c101 - c100, fb, c100), c11 = fmaf(c111 - c110, fb, c110);
+                const float lo = fmaf(c01 - c00, fg, c00), hi = fmaf(c11 - c10, fg, c10);
+                out[c][k] = fmaf(hi - lo, fr, lo);
             }
+        }
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+            if constexpr (VEC == 4)
+                __stcs(reinterpret_cast<float4 *>(y + c * plane) + p,
+                       make_float4(out[c][0], out[c][1], out[c][2], out[c][3]));
+            else
+                __stcs(y + c * plane + p, out[c][0]);
         }
     }
 }
@@ -231,22 +225,23 @@ __global__ void __launch_bounds__(kFitThreads) lut3d_fit2d_kernel(const float *_
 }
 
 // Fewest pixels of an image for the shared-memory gathers: 14 us against 23 at
-// 512 x 512.  One image only: in a batch CTAs load a second table or stay idle
-// (3 photos of 2027 x 1000, D = 33: 65 us against 58 through L1).
+// 512 x 512.  One image only: images after another in one launch load a second
+// table or leave CTAs idle (3 photos of 2027 x 1000, D = 33: 65 us against 58
+// through L1).
 constexpr size_t kMinShared = size_t(1) << 18;
 
 template <int CH, int VEC>
-svdlut_status launch_shared(const float *lut, int D, int B, size_t plane, const float *x, float *y, const DeviceInfo &di,
+svdlut_status launch_shared(const float *lut, int D, size_t plane, const float *x, float *y, const DeviceInfo &di,
                             cudaStream_t s)
 {
     const svdlut_status st = allow_smem_once(reinterpret_cast<const void *>(lut3d_shared_kernel<CH, VEC>),
                                              di.max_smem_optin, di.device);
     if (st != SVDLUT_OK) return st;
-    const size_t units = plane / VEC * B;
+    const size_t units = plane / VEC;
     const int groups = static_cast<int>(std::min<size_t>(std::max(di.sm_count / (3 / CH), 1),
                                                          (units + kSharedThreads - 1) / kSharedThreads));
     lut3d_shared_kernel<CH, VEC><<<groups * (3 / CH), kSharedThreads, sizeof(float) * CH * D * table_strides(D).r, s>>>(
-        lut, D, B, plane, groups, x, y);
+        lut, D, plane, groups, x, y);
     SVDLUT_CUDA_TRY(cudaGetLastError());
     return SVDLUT_OK;
 }
@@ -288,10 +283,10 @@ extern "C" svdlut_status svdlut_lut3d_apply(int D, const float *lut3d, int B, in
     if (B == 1 && plane >= kMinShared && table <= limit && apart) {
         const bool all = 3 * table <= limit, vec = plane % 4 == 0 && aligned(x, 16) && aligned(y, 16);
         if (all)
-            return vec ? launch_shared<3, 4>(lut3d, D, B, plane, x, y, di, s)
-                       : launch_shared<3, 1>(lut3d, D, B, plane, x, y, di, s);
-        return vec ? launch_shared<1, 4>(lut3d, D, B, plane, x, y, di, s)
-                   : launch_shared<1, 1>(lut3d, D, B, plane, x, y, di, s);
+            return vec ? launch_shared<3, 4>(lut3d, D, plane, x, y, di, s)
+                       : launch_shared<3, 1>(lut3d, D, plane, x, y, di, s);
+        return vec ? launch_shared<1, 4>(lut3d, D, plane, x, y, di, s)
+                   : launch_shared<1, 1>(lut3d, D, plane, x, y, di, s);
     }
     float4 *packed = static_cast<float4 *>(ws);
     lut3d_pack_kernel<<<grid_for(static_cast<size_t>(B) * n3, di.sm_count), 256, 0, s>>>(lut3d, B, n3, packed);
