@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) lut3d_apply_kernel(const float4 *__restri
 // pixel and channel, about 3.5 passes each for noise (32 random banks) and 1 to 2
 // for smooth content; a 16-byte gather of the three channels through L1 moves 16
 // bytes for 12 and misses L1 (575 KB) unless the pixels are coherent.  One 4K
-// frame, D = 33: 81 us for half noise, half smooth (113 through L1), 71 for a
+// frame, D = 33: 79 us for half noise, half smooth (113 through L1), 66 for a
 // photo (70).
 constexpr int kSharedThreads = 1024;
 
