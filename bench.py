@@ -37,7 +37,7 @@ N_SETS = 4  # rotating input/output sets: 4 x 199 MB > 129 MB L2
 
 
 KERNEL_SOURCES = ("paper_2508_16121_gb300/csrc/apply_kernel.cuh", "paper_2508_16121_gb300/csrc/apply_launch.cuh",
-                  "paper_2508_16121_gb300/csrc/svdlut_apply.cu")
+                  "paper_2508_16121_gb300/csrc/apply_instances.cuh", "paper_2508_16121_gb300/csrc/svdlut_apply.cu")
 # ncu counters of the headline kernel (dram bytes per launch), with the hash
 # of the kernel sources they were taken on
 PROFILE_COUNTERS = "profiles/apply_kernel_f32_3840x2160_mix.json"
@@ -378,7 +378,7 @@ def run_ours(args, world, rank, local):
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": profiled_traffic(),
                      "limiter": profiled_limiter(),
-                     "kernel": "apply_kernel<Io<InF32, OutF32>, 16, false>",
+                     "kernel": "apply_kernel<Io<InF32, OutF32>, 16, false, kPreAll, true, true>",
                      "timed": "CUDA events around the K back-to-back calls of the timed region, per call "
                               "(prep_kernel + apply_kernel)",
                      "bytes_per_launch": bytes_launch,
