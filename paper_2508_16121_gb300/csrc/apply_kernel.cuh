@@ -1321,8 +1321,12 @@ __host__ __device__ __forceinline__ bool fast_rows(const ImgDesc &d)
 // from every image.  FAST: every image takes fast rows; otherwise each block
 // decides.  Both are template parameters because the pixel loop needs all 128
 // registers: with the table construction and the general rows in the same
-// kernel it spilled, and 4K frames took 100 us instead of 94 (kPreAll alone is
-// small enough for both kinds of rows).
+// kernel it spilled, and 4K frames took 100 us instead of 94.  kPreAll, which
+// those frames and the adjoint take, has no spills with either kind of rows
+// (interleaved 8-bit 12 bytes).  What builds tables beside the general rows or
+// the unaligned accesses still has some, bytes stored / loaded: float kPreNone 72 /
+// 104 with general rows, 8 / 16 with fast aligned ones, kPreFolds unaligned 28 /
+// 44, the adjoint without a workspace 64 to 100 / 80 to 144.
 // VEC: every image allows whole-lane vector accesses (ImgDesc::vec); the code of
 // the unaligned ones costs the aligned frames 1.5 %.
 template <class IO, int N, bool DX, int PRE, bool FAST, bool VEC>

@@ -24,8 +24,6 @@ ImgDesc make_desc_io(const svdlut_dims *d, const svdlut_params *p, int b, int H,
 
 // Shared-memory bytes of args a for block heights up to bh_max; the
 // all-nine-tables prologue is enabled when it fits.  Sets lcell/scratch sizes.
-// Shared-memory bytes of args a for block heights up to bh_max; the
-// all-nine-tables prologue is enabled when it fits.  Sets lcell/scratch sizes.
 template <int N>
 size_t apply_smem_bytes(LaunchArgs<N> &a, size_t limit)
 {

@@ -69,9 +69,10 @@ struct BwdArgs {
 // room for 15 warps and their queues.  Noise, a new cell at every pixel, is
 // bound by the shared-memory pipe (about 85 wavefronts a batch); smooth
 // content by latency and issue slots, photos with pixel noise by the trees.
-// Measured on 8 x 1920x1080, with lut_finalize_kernel: noise 538 us, smooth
-// 287, half and half 429 (710 when each change of a lane's cell was scattered
-// at once, from 12 warps with four floats per vertex).  Also tried: one table
+// Measured on 8 x 1920x1080, with lut_finalize_kernel: noise 534 us, smooth
+// 310, half and half 413 (710 when each change of a lane's cell was scattered
+// at once, from 12 warps with four floats per vertex).  Also tried, with whole
+// CTAs per image, where the present way took 538, 287 and 429: one table
 // of cells (48 bytes at one place, 66 wavefronts a batch) per pair, which its
 // warps update in turns: 660, 440 and 563 us, the hand-over's latency; 12
 // warps of this kernel: 580, 323, 460 us; the queue for every batch: 671,
@@ -1018,8 +1019,6 @@ struct BwdPlan {
 
 static size_t align256(size_t v) { return (v + 255) & ~static_cast<size_t>(255); }
 
-// Lets kernel f use dynamic shared memory up to the opt-in limit minus its
-// static shared memory.
 // Opts kernel f into the largest dynamic shared memory its static shared
 // memory leaves, once per device (calls from several threads are serialised).
 static svdlut_status allow_dynamic_smem(const void *f, int max_optin, int device)
