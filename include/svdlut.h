@@ -364,9 +364,10 @@ svdlut_status svdlut_cie94(const float *y, const float *target, int B, int H, in
  * the same arguments as svdlut_backward minus the workspace; its scratch space
  * is a fixed 32 MiB array inside the library (present on every GPU that loads
  * it, until the process exits), and it allocates nothing.
- *  - Sizes whose svdlut_backward_workspace_size exceeds 32 MiB are rejected
- *    with SVDLUT_ERR_UNSUPPORTED.  The workspace plan depends on the GPU's SM
- *    count; on a 152-SM GB300, 8 x 1920x1080 and one 3840x2160 image (D_t=33,
+ *  - Where svdlut_backward's plan (svdlut_backward_workspace_size) wants more
+ *    than 32 MiB, the fastest plan that fits is taken; sizes with none are
+ *    rejected with SVDLUT_ERR_UNSUPPORTED.  The workspace plan depends on the
+ *    GPU's SM count; on a 152-SM GB300, 8 x 1920x1080 and one 3840x2160 image (D_t=33,
  *    rank 8, K=8 grids at 1/8 resolution) fit.
  *  - The first call on a device looks up the array's device address (one
  *    cudaGetSymbolAddress with that device current); make that first call
